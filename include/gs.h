@@ -131,9 +131,10 @@ typedef struct {            /* zero-initialised = defaults */
                                   the strip kernel (the FP64 saddle operator then uses 32 x 8 tiles);
                                   5 -> by size, the strip kernel on levels of at least 32,768 cells
                                   and 32 x 8 tiles below (no timing at gs_create).
-                               3D meshes: 0 -> time the cell tiles of 8 x 8 x 8 and 8 x 8 x 4
-                                  evaluated cells per level and keep the faster (default);
-                                  2 -> always 8 x 8 x 4; any other value -> always 8 x 8 x 8.
+                               3D meshes: 0 -> time cell-layer segments of the length chosen by size
+                                  and of at most 4 evaluated layers per level and keep the faster
+                                  (default); 2 -> always at most 4 layers; any other value -> always
+                                  by size.
                                   Every variant sums a node's cell contributions in the same order,
                                   so the results do not depend on the choice. */
   int deflate;              /* 1: rigid-body deflation of stiff inclusions in the V-cycle's finest
@@ -339,8 +340,8 @@ typedef struct {
   int pressure_coarse_free;/* unknowns of the dense coarse pressure-Laplacian solve */
   double plambda_max[16];  /* Chebyshev upper bound of the pressure Laplacian per level */
   int tile_rows[16];       /* 2D: evaluated cell rows per tile chosen for each level's multigrid kernels
-                              (0: the strip kernel); 3D: evaluated cell layers along z per 8 x 8 x k
-                              tile (8 or 4) */
+                              (0: the strip kernel); 3D: 4 for segments of at most 4 evaluated cell
+                              layers, 8 for segments of the length chosen by size */
   int saddle_tile_rows;    /* the same for the FP64 saddle operator */
   int deflation_inclusions;/* stiff inclusions in the deflation space (option deflate) */
   int deflation_modes;     /* rigid modes kept (modes vanishing on unconstrained nodes dropped) */

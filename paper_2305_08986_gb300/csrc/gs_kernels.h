@@ -41,26 +41,15 @@ struct TileArgs {
   T rho, ihx, ihy, wq;  // density, 1 / h_x, 1 / h_y, h_x h_y (3D: h_x h_y h_z)
   T ihz;                // 1 / h_z (3D)
   int tiles[3];
-  T* part;        // 3D FP32: per-tile partial sums of the nodes on shared tile faces (gs_tile.cu,
-                  // tile3nh_body; NULL: the halo tiles are used)
   int shape;      // 2D velocity-block variant (0 / 1 / 2: tiles of 16 / 17 / 8 rows of evaluated cells,
                   // 3: the strip kernel of gs_strip2d.cuh; other operator blocks: 3 -> tiles of 8);
-                  // 3D: 0 / 1 -> tiles of 8 x 8 x 8 / 8 x 8 x 4 evaluated cells
+                  // 3D: 0 / 1 -> segments of the length the launcher chooses / at most 4 evaluated layers
 };
 constexpr int kTileShapes2D = 4;   // velocity-block variants the autotuner times
 constexpr int kTileHeights2D = 3;  // tile variants of the full saddle operator
-// 3D cell tiles (TileArgs::shape): 0 -> 8 x 8 x 8, 1 -> 8 x 8 x 4 evaluated cells; every variant
-// sums a node's cell contributions in the same order, so the choice does not change any result
+// 3D march kernel (TileArgs::shape): 0 -> segment length by size, 1 -> at most 4 evaluated cell layers;
+// every node sums its cells in the same order, so the choice does not change any result
 constexpr int kTileShapes3D = 2;
-// FP32 3D velocity block without halo cells (gs_tile.cu, tile3nh_body): tiles of 8 x 8 x 4 cells, a
-// 17 x 17 x 9 node box each; the partial-sum buffer holds 3 boxes (one per component) per tile
-constexpr int kNH3Cells0 = 8, kNH3Cells1 = 8, kNH3Cells2 = 4;
-constexpr int kNH3Box = (2 * kNH3Cells0 + 1) * (2 * kNH3Cells1 + 1) * (2 * kNH3Cells2 + 1);
-inline long long nh3_part_elems(const int n[3]) {
-  const long long t = (long long)((n[0] + kNH3Cells0 - 1) / kNH3Cells0) * ((n[1] + kNH3Cells1 - 1) / kNH3Cells1) *
-                      ((n[2] + kNH3Cells2 - 1) / kNH3Cells2);
-  return t * 3 * kNH3Box;
-}
 constexpr int tile3d_depth(int shape) { return shape == 1 ? 4 : 8; }
 
 // Which blocks of the saddle operator a launch computes.
@@ -70,6 +59,13 @@ template <typename T>
 cudaError_t launch_tile(int dim, int mode, int ops, TileArgs<T> a, cudaStream_t st);
 template <typename T>
 cudaError_t launch_tile2d(int mode, int ops, TileArgs<T> a, cudaStream_t st);
+// 3D (gs_march3d.cuh): the velocity block, B, B^T and the saddle operator without corrector terms
+template <typename T>
+cudaError_t launch_march3d(int mode, int ops, const TileArgs<T>& a, cudaStream_t st);
+template <>
+cudaError_t launch_march3d<float>(int, int, const TileArgs<float>&, cudaStream_t);
+template <>
+cudaError_t launch_march3d<double>(int, int, const TileArgs<double>&, cudaStream_t);
 template <typename T>
 cudaError_t launch_strip2d(int mode, TileArgs<T> a, cudaStream_t st);
 // one CTA whose bounded mbarrier wait runs out (about a second) and sets *err

@@ -1,44 +1,9 @@
 // Launcher of the 2D strip kernel (gs_strip2d.cuh).
-#include <atomic>
-
+#include "gs_occ.cuh"
 #include "gs_strip2d.cuh"
 
 namespace gs {
 namespace {
-
-int device_index() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return -1;
-  return dev;
-}
-
-int sm_count() {
-  static std::atomic<int> cache[kMaxDevices];
-  const int dev = device_index();
-  if (dev >= 0 && cache[dev].load(std::memory_order_relaxed) > 0) return cache[dev].load(std::memory_order_relaxed);
-  int v = 0;
-  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev < 0 ? 0 : dev) != cudaSuccess || v <= 0) v = 1;
-  if (dev >= 0) cache[dev].store(v, std::memory_order_relaxed);
-  return v;
-}
-
-// Resident CTAs per SM of the kernel with `smem` bytes of dynamic shared memory (per device).
-template <class K>
-int ctas_per_sm(size_t smem) {
-  static std::atomic<size_t> enabled[kMaxDevices];
-  static std::atomic<int> cache[kMaxDevices];
-  const int dev = device_index();
-  if (dev >= 0 && cache[dev].load(std::memory_order_relaxed) > 0) return cache[dev].load(std::memory_order_relaxed);
-  int n = 1;
-  if (ensure_dynamic_smem(k_one<K>, smem, enabled) == cudaSuccess &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_one<K>, K::THREADS, smem) == cudaSuccess && n > 0) {
-    if (dev >= 0) cache[dev].store(n, std::memory_order_relaxed);
-  } else {
-    cudaGetLastError();
-    n = 1;
-  }
-  return n;
-}
 
 // Batches per segment: minimise (waves of the grid) x (batches per CTA), then the rows evaluated.
 void choose_segments(int n0, int n1, int slots, int* strips, int* segs, int* nb_out) {
