@@ -120,113 +120,6 @@ __device__ __forceinline__ void sweep(const T* __restrict__ in, T* __restrict__ 
   }
 }
 
-// ---- viscous + mass block -------------------------------------------------------------------
-// y_a = sum_b A_ab^K x_b for both output components a of a 2D cell, with A^K the cell block of
-// alpha (phi_i, phi_j) delta_ab + eta_K (2 eps(phi_j e_b), eps(phi_i e_a)).  Writes y (not +=).
-//
-// Diagonal block (true 1D matrices M, K):  alpha MM + eta (1+[a=x]) K_x M_y + eta (1+[a=y]) M_x K_y;
-// off-diagonal blocks: eta (E^T along x)(E along y) x_y for a = x, eta (E along x)(E^T along y) x_x
-// for a = y.  Evaluation, per input component (three node columns along y):
-//   1. the three sweeps along y that the component feeds (M, K and E or E^T) from the symmetric and
-//      antisymmetric parts s = x_0 + x_2, d = x_0 - x_2 of each column (M and K are centro-symmetric,
-//      E and E^T centro-antisymmetric), e.g. (M x)_0 = 1.5 s + 2.5 d + 2 x_1;
-//   2. per output node row, one fused combination along x, y_row = (mm M + cq K) a + ck M k + ce G r,
-//      again from the symmetric / antisymmetric parts of the swept rows: y_0 = S + D, y_2 = S - D.
-// This takes about 40 % fewer floating-point operations than sweeping each 1D operator separately;
-// the exact 1D matrices are those of the header, only the association of the sums differs.
-template <typename T>
-__device__ __forceinline__ void ysweep_mk(T x0, T x1, T x2, T& s, T& d, T (&m)[3], T (&k)[3], T& q4) {
-  s = x0 + x2;
-  d = x0 - x2;
-  const T q2 = T(2) * x1, q16 = T(16) * x1;
-  q4 = T(4) * x1;
-  const T u = fma(T(1.5), s, q2);          // M = [4 2 -1; 2 16 2; -1 2 4]
-  m[0] = fma(T(2.5), d, u);
-  m[2] = fma(T(-2.5), d, u);
-  m[1] = fma(T(2), s, q16);
-  const T v = fma(T(4), s, T(-2) * q4);    // K = [7 -8 1; -8 16 -8; 1 -8 7]
-  k[0] = fma(T(3), d, v);
-  k[2] = fma(T(-3), d, v);
-  k[1] = fma(T(-8), s, q16);
-}
-
-// Output node row of component a from the swept rows a_ (M_y x_a), k_ (K_y x_a), r_ (the off-diagonal
-// sweep); CA = 0: G = E^T along x (output x), CA = 1: G = E along x (output y).
-template <int CA, typename T>
-__device__ __forceinline__ void xrow_fused(const T* a_, const T* k_, const T* r_, T hs, T hd, T c01, T c11, T ck15,
-                                           T ck2, T ck25, T ck16, T ce, T* y) {
-  const T sa = a_[0] + a_[2], da = a_[0] - a_[2];
-  const T sk = k_[0] + k_[2], dk = k_[0] - k_[2];
-  const T sr = r_[0] + r_[2], dr = r_[0] - r_[2];
-  // S = (y0 + y2) / 2, D = (y0 - y2) / 2
-  T S = hs * sa + c01 * a_[1] + ck15 * sk + ck2 * k_[1];
-  T D = hd * da + ck25 * dk;
-  T y1 = c01 * sa + c11 * a_[1] + ck2 * sk + ck16 * k_[1];
-  if (CA == 0) {  // E^T = [-3 4 -1; -4 0 4; 1 -4 3]
-    S = fma(-ce, dr, S);
-    D = fma(T(-2) * ce, sr, fma(T(4) * ce, r_[1], D));
-    y1 = fma(T(-4) * ce, dr, y1);
-  } else {        // E = [-3 -4 1; 4 0 -4; -1 4 3]
-    S = fma(T(-2) * ce, dr, S);
-    D = fma(-ce, sr, fma(T(-4) * ce, r_[1], D));
-    y1 = fma(T(4) * ce, dr, y1);
-  }
-  y[0] = S + D;
-  y[1] = y1;
-  y[2] = S - D;
-}
-
-template <typename T>
-__device__ __forceinline__ void cell_A2(const T (&x)[2][9], T (&y)[2][9], T eta, const OpCoef<T>& c) {
-  // sweeps along y, column by column (column i = nodes i, i + 3, i + 6)
-  T a[2][9], k[2][9], r[2][9];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    T s0, d0, q40, m0[3], k0[3];
-    ysweep_mk(x[0][i], x[0][i + 3], x[0][i + 6], s0, d0, m0, k0, q40);
-    T s1, d1, q41, m1[3], k1[3];
-    ysweep_mk(x[1][i], x[1][i + 3], x[1][i + 6], s1, d1, m1, k1, q41);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      a[0][i + 3 * j] = m0[j];
-      k[0][i + 3 * j] = k0[j];
-      a[1][i + 3 * j] = m1[j];
-      k[1][i + 3 * j] = k1[j];
-    }
-    // output x takes E_y x_y: E = [-3 -4 1; 4 0 -4; -1 4 3]
-    const T z = s1 + q41;
-    r[0][i] = fma(T(-2), d1, -z);
-    r[0][i + 3] = T(4) * d1;
-    r[0][i + 6] = fma(T(-2), d1, z);
-    // output y takes E^T_y x_x: E^T = [-3 4 -1; -4 0 4; 1 -4 3]
-    r[1][i] = fma(T(-2), s0, q40 - d0);
-    r[1][i + 3] = T(-4) * d0;
-    r[1][i + 6] = fma(T(2), s0, -(d0 + q40));
-  }
-  const T mm = c.mm;
-  const T ce = eta * c.ex[0];
-#pragma unroll
-  for (int comp = 0; comp < 2; ++comp) {
-    const T ck = (comp == 1 ? T(2) : T(1)) * eta * c.km[1];   // stiffness along y
-    const T cq = (comp == 0 ? T(2) : T(1)) * eta * c.km[0];   // stiffness along x
-    // C = mm M + cq K: c00 = 4 mm + 7 cq, c01 = 2 mm - 8 cq, c02 = cq - mm, c11 = 16 (mm + cq)
-    const T hs = fma(T(1.5), mm, T(4) * cq);   // (c00 + c02) / 2
-    const T hd = fma(T(2.5), mm, T(3) * cq);   // (c00 - c02) / 2
-    const T c01 = fma(T(2), mm, T(-8) * cq);
-    const T c11 = T(16) * (mm + cq);
-    const T ck15 = T(1.5) * ck, ck2 = T(2) * ck, ck25 = T(2.5) * ck, ck16 = T(16) * ck;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      if (comp == 0)
-        xrow_fused<0>(a[0] + 3 * j, k[0] + 3 * j, r[0] + 3 * j, hs, hd, c01, c11, ck15, ck2, ck25, ck16, ce,
-                      y[0] + 3 * j);
-      else
-        xrow_fused<1>(a[1] + 3 * j, k[1] + 3 * j, r[1] + 3 * j, hs, hd, c01, c11, ck15, ck2, ck25, ck16, ce,
-                      y[1] + 3 * j);
-    }
-  }
-}
-
 // ---- corrector stage: convection by a given field and streamline diffusion (2D) -----------------
 // In the corrector stage (Sec. 3.1.2, Eq. "v_star") the velocity block gains
 //   rho ((v° . grad) u, w)                                   (convection by the given Q2 field v°)
@@ -452,32 +345,6 @@ __device__ __forceinline__ void sweep_w(const T* __restrict__ in, const int* ro,
       }
     }
   }
-}
-
-// ---- divergence block B and its transpose -----------------------------------------------------
-// (B u)_q = - sum_b int psi_q d phi_j/dx_b u_jb :  -sum_b (G in direction b, N elsewhere) u_b
-template <typename T>
-__device__ __forceinline__ void cell_B2(const T (&u)[2][9], T (&out)[4], const OpCoef<T>& c) {
-  T t[6], s[4];
-  sweep<OpN, 1, 3, 3, 1, false>(u[0], t);  // (3,2)
-  sweep<OpG, 0, 3, 2, 1, false>(t, out);   // (2,2)
-  sweep<OpG, 1, 3, 3, 1, false>(u[1], t);
-  sweep<OpN, 0, 3, 2, 1, false>(t, s);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) out[i] = -(c.bd[0] * out[i] + c.bd[1] * s[i]);
-}
-
-template <typename T>
-__device__ __forceinline__ void cell_BT2(const T (&p)[4], T (&u)[2][9], const OpCoef<T>& c, bool acc) {
-  T t[6], v[9];
-  sweep<OpNT, 1, 2, 2, 1, false>(p, t);  // (2,3)
-  sweep<OpGT, 0, 2, 3, 1, false>(t, v);  // (3,3)
-#pragma unroll
-  for (int i = 0; i < 9; ++i) u[0][i] = (acc ? u[0][i] : T(0)) - c.bd[0] * v[i];
-  sweep<OpGT, 1, 2, 2, 1, false>(p, t);
-  sweep<OpNT, 0, 2, 3, 1, false>(t, v);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) u[1][i] = (acc ? u[1][i] : T(0)) - c.bd[1] * v[i];
 }
 
 // ---- 3D operator in a rotated frame: one code path for every output component ------------------

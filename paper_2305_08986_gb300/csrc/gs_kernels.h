@@ -19,6 +19,7 @@ template <typename T>
 struct TileArgs {
   Geom g;
   OpCoef<T> c;
+  Modal2<T> m2;   // 2D: coefficients in the cells' modes (set by the launcher)
   const T* eta;   // per cell
   const T* alpha; // per cell factor of the mass term (alpha_K; NULL: 1, alpha then lives in c.mm)
   const T* xu;    // velocity input (A and B), CHEB: current iterate

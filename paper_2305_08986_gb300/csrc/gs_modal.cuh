@@ -108,6 +108,104 @@ __device__ __forceinline__ void plane_from_modes(T (&v)[9]) {
   for (int j = 0; j < 3; ++j) from_modes(v[3 * j], v[3 * j + 1], v[3 * j + 2], v[3 * j], v[3 * j + 1], v[3 * j + 2]);
 }
 
+// product kept apart from the sums around it (a contraction there could differ from kernel to kernel)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// position of a 2D mode (i, j) in Modal2::dm (symmetric in i and j)
+__host__ __device__ constexpr int modal2_class(int i, int j) {
+  const int lo = i < j ? i : j, hi = i < j ? j : i;
+  return lo == 0 ? hi : (lo == 1 ? 2 + hi : 5);
+}
+
+template <typename T>
+inline Modal2<T> make_modal2(const Geom& g, const OpCoef<T>& c) {
+  const ModalCoef<T> m = make_modal<T>(g, c);
+  Modal2<T> q{};
+  for (int j = 0; j < 3; ++j)
+    for (int i = 0; i < 3; ++i) {
+      q.dm[modal2_class(i, j)] = m.dm[modal_class(i, j, 0)];
+      for (int a = 0; a < 2; ++a) q.dk[a][i + 3 * j] = m.dk[a][i + 3 * j];
+    }
+  for (int a = 0; a < 2; ++a) {
+    q.g2[a] = m.g2[a];
+    q.g3[a] = m.g3[a];
+    q.g23[a] = m.g23[a];
+  }
+  return q;
+}
+
+// One 2D cell: y = (alpha_K M + eta_K viscous) x + B^T p, pb = B x (nodal values in and out; the blocks
+// by the flags), every sum in the cell's modes.  alpha: factor of the mass term (alpha_K or 1).
+template <bool WA, bool WBT, bool WB, typename T>
+__device__ __forceinline__ void cell_modal2(const T (&x)[2][9], const T (&p)[4], T (&y)[2][9], T (&pb)[4], T eta, T alpha,
+                                            const Modal2<T>& m) {
+  T a[2][9], r[2][9];
+  if (WA || WB) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+#pragma unroll
+      for (int q = 0; q < 9; ++q) a[c][q] = x[c][q];
+      plane_to_modes(a[c]);
+    }
+  }
+  if (WA) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const T ms = mul_rn(alpha, m.dm[modal2_class(q % 3, q / 3)]);
+        r[c][q] = mul_rn(q == 0 ? ms : fma(eta, m.dk[c][q], ms), a[c][q]);
+      }
+    // coupling: mode (0|1, 1|2) of component x with (+1, -1) of component y, products E E = 1/36, ...
+    const T g1 = mul_rn(eta, T(1.0 / 36.0)), g2 = T(2) * g1, g4 = T(4) * g1, g8 = T(8) * g1;
+    r[0][3] = fma(g1, a[1][1], r[0][3]);
+    r[1][1] = fma(g1, a[0][3], r[1][1]);
+    r[0][6] = fma(g4, a[1][4], r[0][6]);
+    r[1][4] = fma(g2, a[0][6], r[1][4]);
+    r[0][4] = fma(g2, a[1][2], r[0][4]);
+    r[1][2] = fma(g4, a[0][4], r[1][2]);
+    r[0][7] = fma(g8, a[1][5], r[0][7]);
+    r[1][5] = fma(g8, a[0][7], r[1][5]);
+  } else if (WBT) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int q = 0; q < 9; ++q) r[c][q] = T(0);
+  }
+  if (WBT) {
+    const T s0 = p[0] + p[1], d0 = p[1] - p[0], s1 = p[2] + p[3], d1 = p[3] - p[2];
+    const T b00 = s0 + s1, b10 = d0 + d1, b01 = s1 - s0, b11 = d1 - d0;
+    r[0][1] = fma(-m.g2[0], b00, r[0][1]);
+    r[0][4] = fma(-m.g2[0], b01, r[0][4]);
+    r[0][2] = fma(-m.g23[0], b10, r[0][2]);
+    r[0][5] = fma(-m.g23[0], b11, r[0][5]);
+    r[1][3] = fma(-m.g2[1], b00, r[1][3]);
+    r[1][4] = fma(-m.g2[1], b10, r[1][4]);
+    r[1][6] = fma(-m.g23[1], b01, r[1][6]);
+    r[1][7] = fma(-m.g23[1], b11, r[1][7]);
+  }
+  if (WA || WBT) {
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      plane_from_modes(r[c]);
+#pragma unroll
+      for (int q = 0; q < 9; ++q) y[c][q] = r[c][q];
+    }
+  }
+  if (WB) {
+    const T c00 = fma(-m.g2[0], a[0][1], mul_rn(-m.g2[1], a[1][3]));
+    const T c01 = fma(-m.g2[0], a[0][4], mul_rn(-m.g3[1], a[1][6]));
+    const T c10 = fma(-m.g3[0], a[0][2], mul_rn(-m.g2[1], a[1][4]));
+    const T c11 = fma(-m.g3[0], a[0][5], mul_rn(-m.g3[1], a[1][7]));
+    const T s0 = c00 - c01, s1 = c00 + c01, d0 = c10 - c11, d1 = c10 + c11;  // y = 0 / 1: modes along x
+    pb[0] = s0 - d0;
+    pb[1] = s0 + d0;
+    pb[2] = s1 - d1;
+    pb[3] = s1 + d1;
+  }
+}
+
 // r = (alpha_K M + eta_K viscous) a in the modes of one 3D cell; mass: the alpha_K-scaled dm
 template <typename T>
 __device__ __forceinline__ void modal_A3(const T (&a)[3][27], T (&r)[3][27], T eta, const T (&mass)[10],

@@ -22,6 +22,8 @@
 // alpha, constraint mask) of batch k + 1 is loaded into registers during batch k.
 // Every mbarrier wait is bounded: a wait that gives up sets TileArgs::err and the launch completes.
 //
+// Cells are evaluated in their Legendre modes (gs_modal.cuh, ~150 operations).
+//
 // Sums.  A cell's 18 results (9 nodes x 2 components) are reduced without a shared-memory round
 // trip per cell: the left node column of a cell receives the right column of the cell to its left
 // by a warp shuffle, and the bottom node row receives the top row of the cells below and below-left
@@ -36,8 +38,7 @@
 #pragma once
 #include <stdint.h>
 
-#include "gs_cell.cuh"
-#include "gs_kernels.h"
+#include "gs_modal.cuh"
 
 namespace gs {
 namespace strip2d {
@@ -263,21 +264,20 @@ __device__ __forceinline__ void strip2d_body(const TileArgs<T>& A, int bid) {
   struct CellData {
     T eta, alpha;
     unsigned cmv;  // constrained local nodes (bits 0..8), obstacle cell (bit 15)
-    int cell;
     bool inmesh;
   };
   auto load_cell = [&](int k) {
     CellData d;
     const int c0 = cs0 - 1 + lane, c1 = r0 - 1 + NW * k + w;
     d.inmesh = c0 >= 0 && c0 < n0 && c1 >= 0 && c1 < n1;
-    d.cell = d.inmesh ? c0 + n0 * c1 : 0;
+    const int cell = d.inmesh ? c0 + n0 * c1 : 0;
     d.cmv = 0;
     d.eta = T(0);
     d.alpha = T(1);
     if (d.inmesh) {
-      d.cmv = g.ccmask ? (unsigned)g.ccmask[d.cell] : face_cell_mask(g, c0, c1);
-      d.eta = A.eta[d.cell];
-      if (A.alpha) d.alpha = A.alpha[d.cell];
+      d.cmv = g.ccmask ? (unsigned)g.ccmask[cell] : face_cell_mask(g, c0, c1);
+      d.eta = A.eta[cell];
+      if (A.alpha) d.alpha = A.alpha[cell];
     }
     return d;
   };
@@ -301,7 +301,6 @@ __device__ __forceinline__ void strip2d_body(const TileArgs<T>& A, int bid) {
     const int t = NW * k + w;          // processed row index within the segment (0: halo row)
     const int c0 = cs0 - 1 + lane, c1 = r0 - 1 + t;
     const bool inmesh = cur.inmesh;
-    const int cell = cur.cell;
     const unsigned cmv = cur.cmv;
     const unsigned cm = raw ? 0u : (cmv & 0x1FFu);
     const bool active = inmesh && !(cmv & 0x8000u) && cm != 0x1FFu;
@@ -321,8 +320,6 @@ __device__ __forceinline__ void strip2d_body(const TileArgs<T>& A, int bid) {
     for (int i = 0; i < 9; ++i) y[0][i] = y[1][i] = T(0);
     if (active) {
       const T eta = cur.eta * c.eta_scale;
-      OpCoef<T> cK = c;
-      if (A.alpha) cK.mm = c.mm * cur.alpha;
       T xl[2][9];
 #pragma unroll
       for (int comp = 0; comp < 2; ++comp)
@@ -335,7 +332,8 @@ __device__ __forceinline__ void strip2d_body(const TileArgs<T>& A, int bid) {
         for (int i = 0; i < 9; ++i)
           if ((cm >> i) & 1u) xl[0][i] = xl[1][i] = T(0);
       }
-      cell_A2(xl, y, eta, cK);
+      T pl[4], pb[4];
+      cell_modal2<true, false, false>(xl, pl, y, pb, eta, cur.alpha, A.m2);
     }
     // top node row, unreduced, to the warp above (warp NW - 1: to warp 0 of the next batch, which
     // reads it after the next barrier (A)); slots alternate with the batch parity, and a warp can
@@ -441,7 +439,10 @@ __device__ __forceinline__ void strip2d_body(const TileArgs<T>& A, int bid) {
 template <typename T, int MODE>
 struct Strip2dK {
   using Args = TileArgs<T>;
-  static constexpr int THREADS = NT, MINB = sizeof(T) == 4 ? 3 : 1;
+  // FP32 A x needs 64 registers with the cells in Legendre modes and runs 4 CTAs per SM: 10.2 -> 7.8 us on
+  // 1280 x 210 cells (11.5 us before); the residual and the Chebyshev step, with their operand windows,
+  // stay at 3 (a smoother call of four steps on 1280 x 224: 85.2 us, 86.5 us at 4, 90.7 us before)
+  static constexpr int THREADS = NT, MINB = sizeof(T) == 4 ? (MODE == TILE_APPLY ? 4 : 3) : 1;
   static __device__ __forceinline__ void body(const Args& a, int blk, int) { strip2d_body<T, MODE>(a, blk); }
 };
 

@@ -9,8 +9,9 @@
 //      component), and the epilogue's b / d / D^-1 of the owned nodes, are copied to shared
 //      memory with cp.async (zero fill for nodes outside the mesh and constrained columns), so
 //      all global loads of the CTA are in flight together;
-//   2. every evaluated cell is computed (sum-factorised, gs_cell.cuh) from shared memory and
-//      its 18 velocity (and 4 pressure) results are stored cell-major in shared memory;
+//   2. every evaluated cell is computed in its Legendre modes (gs_modal.cuh) from shared memory, A, B^T
+//      and B together, and its 18 velocity (and 4 pressure) results are stored cell-major in shared
+//      memory;
 //   3. each owned node sums the <= 4 cell results that touch it, in a fixed order (so the
 //      result does not depend on scheduling), and applies the mode's epilogue.
 // Threads form a 32 x 8 grid.  In phases 1 and 3 thread (tx, ty) handles node columns 2 tx and
@@ -18,7 +19,7 @@
 // arithmetic, uniform branches within a warp) and it consumes the epilogue operands it staged.
 #pragma once
 #include "gs_cell.cuh"
-#include "gs_kernels.h"
+#include "gs_modal.cuh"
 
 namespace gs {
 
@@ -267,10 +268,7 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) ob[i] = T(0);
     if (active) {
-      const T eta = A.eta[cell] * c.eta_scale;
-      OpCoef<T> cK = c;  // the cell's mass coefficient (alpha per cell)
-      if (A.alpha) cK.mm = c.mm * A.alpha[cell];
-      T xl[2][9];
+      T xl[2][9], pl[4];
       if (NEED_U) {
         const T* s0p = sx + 2 * e0 + IN0 * 2 * e1;
 #pragma unroll
@@ -281,30 +279,27 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
             xl[1][la + 3 * lb] = s0p[NIN + la + IN0 * lb];
           }
       }
-      if (WA) {
-        cell_A2(xl, yl, eta, cK);
-        if (CONV) {
-          T vl[2][9];
-          const T* v0p = sv + 2 * e0 + IN0 * 2 * e1;
-#pragma unroll
-          for (int lb = 0; lb < 3; ++lb)
-#pragma unroll
-            for (int la = 0; la < 3; ++la) {
-              vl[0][la + 3 * lb] = v0p[la + IN0 * lb];
-              vl[1][la + 3 * lb] = v0p[NIN + la + IN0 * lb];
-            }
-          cell_conv2<CONV>(xl, vl, A.rho, A.rk[cell], A.ihx, A.ihy, A.wq, yl);
-        }
-      }
       if (WBT) {
-        T pl[4];
 #pragma unroll
         for (int lb = 0; lb < 2; ++lb)
 #pragma unroll
           for (int la = 0; la < 2; ++la) pl[la + 2 * lb] = sp[(e0 + la) + PI0 * (e1 + lb)];
-        cell_BT2(pl, yl, c, WA);
       }
-      if (WB) cell_B2(xl, ob, c);
+      const T eta = WA ? A.eta[cell] * c.eta_scale : T(0);
+      const T alpha = WA && A.alpha ? A.alpha[cell] : T(1);
+      cell_modal2<WA, WBT, WB>(xl, pl, yl, ob, eta, alpha, A.m2);
+      if (CONV && WA) {
+        T vl[2][9];
+        const T* v0p = sv + 2 * e0 + IN0 * 2 * e1;
+#pragma unroll
+        for (int lb = 0; lb < 3; ++lb)
+#pragma unroll
+          for (int la = 0; la < 3; ++la) {
+            vl[0][la + 3 * lb] = v0p[la + IN0 * lb];
+            vl[1][la + 3 * lb] = v0p[NIN + la + IN0 * lb];
+          }
+        cell_conv2<CONV>(xl, vl, A.rho, A.rk[cell], A.ihx, A.ihy, A.wq, yl);
+      }
     }
     if (WU) {
 #pragma unroll
@@ -391,8 +386,9 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
 template <typename T, int EY, int MODE, bool WA, bool WBT, bool WB, int CONV = 0>
 struct Tile2dK {
   using Args = TileArgs<T>;
-  // FP64 with B^T (the saddle operator): 3 CTAs per SM (85 registers, a few spills) measured 2.6 %
-  // faster than 2 on the FP64-pipe-bound saddle operator; the FP32 variants stay at 2 (72 registers)
+  // FP64 with B^T (the saddle operator, FP64-pipe-bound): 3 CTAs per SM (76 registers).  1280 x 224: 138 us
+  // with the cells in Legendre modes (~180 FP64 operations per cell), 260 us in 3 x 3 sweeps (~400); the
+  // FP32 variants stay at 2
   static constexpr int THREADS = NT, MINB = CONV ? 1 : (sizeof(T) == 8 && WBT ? 3 : 2);
   static __device__ __forceinline__ void body(const Args& a, int blk, int) {
     tile2d_body<T, EY, MODE, WA, WBT, WB, CONV>(a, blk);
