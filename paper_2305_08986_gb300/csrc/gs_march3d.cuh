@@ -14,6 +14,11 @@
 // sums its cells as ((own + left) + below) + below-left, each term already holding the layer below,
 // so the result does not depend on the patch or segment shape.
 //
+// The patches cover one more column than there are cells along x and y: its threads evaluate nothing and write the
+// mesh's last node lines from their neighbours' contributions, like any other node.  Written by the last cells
+// instead, those lines took a serial chain of loads and stores in a few CTAs, which the whole launch waited for
+// (SMs busy 61 % of the time; 64^3, 4 Chebyshev steps, FP32: 453 -> 318 us; FP64 saddle 37 x 29 x 41: 225 -> 210 us).
+//
 // Every cell of the interior is evaluated once plus the overlap, and nothing is staged: the 27 + 27 node
 // values a thread reads per layer are shared with its neighbours through L1.
 #pragma once
@@ -34,7 +39,7 @@ namespace march3 {
 template <typename T>
 struct Cfg {
   static constexpr int NT = 128;   // threads per CTA
-  static constexpr int MINB = 2;   // CTAs per SM: 8 warps at 255 registers; 12 at 168 spilled (549 against 447 us, 4 Chebyshev steps, 64^3)
+  static constexpr int MINB = 2;   // CTAs per SM: 8 warps at 255 registers; 12 at 168 spilled (4 Chebyshev steps, 64^3: 23 % slower)
 };
 
 // values per thread: exchanged with the neighbours per layer; epilogue operands of the 8 nodes a cell owns
@@ -48,16 +53,13 @@ template <typename T>
 __device__ __forceinline__ T* at(T* base, unsigned off) {
   return reinterpret_cast<T*>(reinterpret_cast<uintptr_t>(base) + off);
 }
-// Asynchronous copies of two consecutive elements of a node row into two value slots of this thread.
+// Asynchronous copies of an element of a node row and, with `two`, its successor into value slots of this thread.
 template <typename T, int SLOT>
-__device__ __forceinline__ void cp_async2(unsigned smem, const T* gmem) {
+__device__ __forceinline__ void cp_async2(unsigned smem, const T* gmem, bool two) {
   constexpr int S = (int)sizeof(T);
-  if (S == 4)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n cp.async.ca.shared.global [%0+%2], [%1+4], 4;\n" ::"r"(smem),
-                 "l"(gmem), "n"(SLOT * S) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n cp.async.ca.shared.global [%0+%2], [%1+8], 8;\n" ::"r"(smem),
-                 "l"(gmem), "n"(SLOT * S) : "memory");
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %2, 0;\n cp.async.ca.shared.global [%0], [%1], %4;\n"
+               " @p cp.async.ca.shared.global [%0+%3], [%1+%4], %4;\n}\n" ::"r"(smem), "l"(gmem), "r"((unsigned)two),
+               "n"(SLOT * S), "n"(S) : "memory");
 }
 
 template <typename T, int MODE, bool WA, bool WBT, bool WB>
@@ -79,31 +81,39 @@ __device__ __forceinline__ void body(const March3Args<T>& M, int bid) {
   const int p0 = bid % M.np0, p1 = (bid / M.np0) % M.np1, sg = bid / (M.np0 * M.np1);
   const int tx = tid % PX, ty = tid / PX;
   const int c0 = p0 * (PX - 1) + tx, c1 = p1 * (M.py - 1) + ty;
-  const bool in = ty < M.py && c0 < n0 && c1 < n1;
+  const bool here = ty < M.py && c0 <= n0 && c1 <= n1;  // c0 = n0, c1 = n1: the mesh's last node lines
+  const bool in = here && c0 < n0 && c1 < n1;           // a cell of the mesh
   const bool left = tx > 0, below = ty > 0;       // neighbours in the patch
-  const bool own = in && (left || p0 == 0) && (below || p1 == 0);
-  const bool lastx = c0 == n0 - 1, lasty = c1 == n1 - 1;
+  const bool own = here && (left || p0 == 0) && (below || p1 == 0);
+  const bool two0 = c0 < n0, two1 = c1 < n1;      // node columns / rows owned besides the first
   const int zs = sg * (M.layers - 1), ze = min(n2, zs + M.layers);
-  // the column's node (0, 0) in a plane (threads outside the mesh read some column of it)
-  const long long vcol = 2 * min(c0, n0 - 1) + (long long)nv0 * (2 * min(c1, n1 - 1));
-  unsigned orow[3];  // byte offsets of its three node rows in a plane (planes are below 4 GB)
+  // byte offsets in a plane (planes are below 4 GB): the cell's three node rows (threads without a cell read some
+  // cell of the mesh), and the two node rows a thread writes
+  const long long vcol = 2 * min(c0, n0) + (long long)nv0 * (2 * min(c1, n1));
+  unsigned orow[3], wrow[2];
+  {
+    const long long rcol = 2 * min(c0, n0 - 1) + (long long)nv0 * (2 * min(c1, n1 - 1));
 #pragma unroll
-  for (int j = 0; j < 3; ++j) orow[j] = (unsigned)((vcol + (long long)nv0 * j) * (long long)sizeof(T));
+    for (int j = 0; j < 3; ++j) orow[j] = (unsigned)((rcol + (long long)nv0 * j) * (long long)sizeof(T));
+#pragma unroll
+    for (int j = 0; j < 2; ++j) wrow[j] = (unsigned)((vcol + (long long)nv0 * j) * (long long)sizeof(T));
+  }
   const long long pcol = c0 + (long long)np0 * c1;
 
   // constrained local nodes of a node plane (bit la + 3 lb)
   unsigned fxy = 0;
   if ((g.faces & 1u) && c0 == 0) fxy |= 0x049u;
-  if ((g.faces & 2u) && lastx) fxy |= 0x124u;
+  if ((g.faces & 2u) && c0 >= n0 - 1) fxy |= c0 == n0 ? 0x049u : 0x124u;
   if ((g.faces & 4u) && c1 == 0) fxy |= 0x007u;
-  if ((g.faces & 8u) && lasty) fxy |= 0x1C0u;
+  if ((g.faces & 8u) && c1 >= n1 - 1) fxy |= c1 == n1 ? 0x007u : 0x1C0u;
   auto plane_mask = [&](int K) -> unsigned {
-    if (!in || raw) return 0u;
+    if (!here || raw) return 0u;
     if (g.vmask) {
       unsigned m = 0;
       const uint8_t* vm = g.vmask + vplane * K + vcol;
 #pragma unroll
-      for (int q = 0; q < 9; ++q) m |= vm[q % 3 + nv0 * (q / 3)] ? 1u << q : 0u;
+      for (int q = 0; q < 9; ++q)
+        if ((two0 || q % 3 == 0) && (two1 || q / 3 == 0)) m |= vm[q % 3 + nv0 * (q / 3)] ? 1u << q : 0u;
       return m;
     }
     if (((g.faces & 16u) && K == 0) || ((g.faces & 32u) && K == 2 * n2)) return 0x1FFu;
@@ -185,13 +195,14 @@ __device__ __forceinline__ void body(const March3Args<T>& M, int bid) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {  // node rows: plane j >> 1, row j & 1
           if (j >= 2 && c2 == n2) break;
+          if ((j & 1) && !two1) continue;
           const long long base = c * Nv + vplane * (2 * c2 + (j >> 1));
           const unsigned o = so32 + (c * 8 + 2 * j) * NT * (unsigned)sizeof(T);
-          cp_async2<T, NT>(o, at(A.bu + base, orow[j & 1]));
+          cp_async2<T, NT>(o, at(A.bu + base, wrow[j & 1]), two0);
           if (ED) {
-            cp_async2<T, NT>(o + 24 * NT * sizeof(T), at(A.dinv + base, orow[j & 1]));
-            cp_async2<T, NT>(o + 72 * NT * sizeof(T), at(A.xu + base, orow[j & 1]));
-            if (A.use_d) cp_async2<T, NT>(o + 48 * NT * sizeof(T), at((const T*)A.d + base, orow[j & 1]));
+            cp_async2<T, NT>(o + 24 * NT * sizeof(T), at(A.dinv + base, wrow[j & 1]), two0);
+            cp_async2<T, NT>(o + 72 * NT * sizeof(T), at(A.xu + base, wrow[j & 1]), two0);
+            if (A.use_d) cp_async2<T, NT>(o + 48 * NT * sizeof(T), at((const T*)A.d + base, wrow[j & 1]), two0);
           }
         }
     }
@@ -321,7 +332,9 @@ __device__ __forceinline__ void body(const March3Args<T>& M, int bid) {
 #pragma unroll
             for (int c = 0; c < 3; ++c)
 #pragma unroll
-              for (int q = 0; q < 4; ++q) xin[c][q] = ldg(at(A.xu + (c * Nv + vplane * (2 * c2 + pl)), orow[q >> 1]) + (q & 1));
+              for (int q = 0; q < 4; ++q)
+                if ((two0 || !(q & 1)) && (two1 || q < 2))
+                  xin[c][q] = ldg(at(A.xu + (c * Nv + vplane * (2 * c2 + pl)), wrow[q >> 1]) + (q & 1));
           }
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
@@ -330,12 +343,10 @@ __device__ __forceinline__ void body(const March3Args<T>& M, int bid) {
             if (left) {
               v[0] += s[-1];
               v[3] += s[NT - 1];
-              if (lasty) v[6] += s[2 * NT - 1];
             }
             if (below) {
               v[0] += s[3 * NT - PX];
               v[1] += s[4 * NT - PX];
-              if (lastx) v[2] += s[2 * NT - PX];
             }
             if (left && below) v[0] += s[2 * NT - PX - 1];
 #pragma unroll
@@ -362,55 +373,22 @@ __device__ __forceinline__ void body(const March3Args<T>& M, int bid) {
           for (int c = 0; c < 3; ++c)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
+              if ((!two0 && (q & 1)) || (!two1 && q >= 2)) continue;
               const long long base = c * Nv + vplane * (2 * c2 + pl);
-              at(y + base, orow[q >> 1])[q & 1] = out[c][q];
-              if (ED) at(A.d + base, orow[q >> 1])[q & 1] = od[c][q];
+              at(y + base, wrow[q >> 1])[q & 1] = out[c][q];
+              if (ED) at(A.d + base, wrow[q >> 1])[q & 1] = od[c][q];
             }
-          if (lastx || lasty) {  // the mesh's right and top boundary nodes
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const T (&v)[9] = pl == 0 ? bot[c] : mid[c];
-#pragma unroll
-              for (int q = 0; q < 9; ++q) {
-                if (q % 3 < 2 && q / 3 < 2) continue;
-                if ((q % 3 == 2 && !lastx) || (q / 3 == 2 && !lasty)) continue;
-                const long long gi = c * Nv + vplane * (2 * c2 + pl) + vcol + q % 3 + nv0 * (q / 3);
-                const bool con = (pm >> q) & 1u;
-                const T ax = con ? (WA ? A.xu[gi] : T(0)) : v[q];
-                if (MODE == TILE_APPLY) {
-                  A.yu[gi] = ax;
-                } else if (MODE == TILE_RESID) {
-                  A.yu[gi] = A.bu[gi] - ax;
-                } else {
-                  T dn = A.c2 * A.dinv[gi] * (A.bu[gi] - ax);
-                  if (A.use_d) dn += A.c1 * A.d[gi];
-                  A.d[gi] = dn;
-                  A.xout[gi] = A.xu[gi] + dn;
-                }
-              }
-            }
-          }
         }
       }
       if (WB) {
         const T* s = slot + (NX - 3) * NT;
-        if (left) {
-          pv[0] += s[-1];
-          if (lasty) pv[2] += s[2 * NT - 1];
-        }
-        if (below) {
-          pv[0] += s[NT - PX];
-          if (lastx) pv[1] += s[2 * NT - PX];
-        }
+        if (left) pv[0] += s[-1];
+        if (below) pv[0] += s[NT - PX];
         if (left && below) pv[0] += s[2 * NT - PX - 1];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (((q & 1) && !lastx) || ((q >> 1) && !lasty)) continue;
-          const long long i = pcol + pplane * c2 + (q & 1) + np0 * (q >> 1);
-          const bool con = !raw && pnode_constrained(g, i);
-          const T bx = con ? (WBT ? A.xp[i] : T(0)) : pv[q];
-          A.yp[i] = MODE == TILE_RESID ? A.bp[i] - bx : bx;
-        }
+        const long long i = pcol + pplane * c2;
+        const bool con = !raw && pnode_constrained(g, i);
+        const T bx = con ? (WBT ? A.xp[i] : T(0)) : pv[0];
+        A.yp[i] = MODE == TILE_RESID ? A.bp[i] - bx : bx;
       }
     }
     pmb = cmt;

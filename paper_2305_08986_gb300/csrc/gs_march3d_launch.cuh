@@ -6,7 +6,7 @@
 namespace gs {
 namespace march3 {
 
-// Patch and segment shape for a mesh of n cells.  Patches of px x py <= NT threads covering an axis of n
+// Patch and segment shape for a mesh of `cells` cells.  Patches of px x py <= NT threads covering an axis of n
 // cells with overlap 1 number ceil((n - 1) / (px - 1)); px is then shrunk to the least that gives that
 // number.  For every patch shape the segments are cut so that the grid is one, two or three waves of the
 // resident CTAs (or single layers, where that is less), and the shape with the least estimated time is
@@ -18,7 +18,8 @@ inline int cover(int n, int p) { return n <= p ? 1 : (n - 1 + p - 2) / (p - 1); 
 inline int shrink(int n, int k) { return k == 1 ? n : (n - 1 + k - 1) / k + 1; }
 
 template <typename T>
-Shape choose(const int* n, int sms, int resident, int max_layers) {
+Shape choose(const int* cells, int sms, int resident, int max_layers) {
+  const int n[3] = {cells[0] + 1, cells[1] + 1, cells[2]};  // the columns of the last node lines included
   const double kShare = sizeof(T) == 4 ? 0.5 : 0.9;
   Shape best{};
   double best_cost = 0.0;
@@ -29,8 +30,8 @@ Shape choose(const int* n, int sms, int resident, int max_layers) {
     s.px = shrink(n[0], s.np0);
     if (s.px > q || s.px < 1) continue;
     const int pymax = Cfg<T>::NT / s.px;
-    if (pymax < 2 && n[1] > 1) continue;
-    s.np1 = cover(n[1], pymax < 2 ? 2 : pymax);
+    if (pymax < 2) continue;
+    s.np1 = cover(n[1], pymax);
     s.py = shrink(n[1], s.np1);
     if (s.px * s.py > Cfg<T>::NT) continue;
     const int patches = s.np0 * s.np1;
