@@ -126,7 +126,8 @@ typedef struct {            /* zero-initialised = defaults */
   int tile_autotune;        /* 2D meshes: 0 -> at gs_create, time each compiled variant of the
                                   velocity-block kernel on every level (cell tiles of 32 x 16,
                                   32 x 17, 32 x 8 evaluated cells; the strip kernel, 31-cell column
-                                  strips marching up row segments) and keep the fastest (default);
+                                  strips marching up row segments; on levels of at most 131,072
+                                  cells also 8 x 8 tiles) and keep the fastest (default);
                                   1 / 2 / 3 -> always the 32 x 16 / 32 x 17 / 32 x 8 tile; 4 -> always
                                   the strip kernel (the FP64 saddle operator then uses 32 x 8 tiles);
                                   5 -> by size, the strip kernel on levels of at least 32,768 cells

@@ -1251,26 +1251,28 @@ gs_status autotune(gs_ctx* c) {
     CK(cudaMemsetAsync(lv.d, 0, sizeof(T) * lv.nu, c->st));
     double best_us = 0.0;
     int best = 0;
-    for (int s = 0; s < nshape; ++s) {
+    const bool small = c->dim == 2 && lv.Nc <= kTileSmallCells;
+    for (int s = 0; s < nshape + small; ++s) {
       TileArgs<T> a = tile_args<T>(lv);
-      a.shape = s;
+      a.shape = s < nshape ? s : kTileSmall2D;
       a.xu = (const T*)lv.xA; a.bu = (const T*)lv.b; a.d = (T*)lv.d; a.dinv = (const T*)lv.dinv;
       a.xout = (T*)lv.xB; a.c1 = (T)0.5; a.c2 = (T)1; a.use_d = 1;
       double us;
       CKS(time_launches(c, [&]() { return launch_tile<T>(c->dim, TILE_CHEB, OPS_A, a, c->st); }, 4, &us));
-      if (s == 0 || us < 0.98 * best_us) { best_us = us; best = s; }
+      if (s == 0 || us < 0.98 * best_us) { best_us = us; best = a.shape; }
     }
     lv.shape = best;
   }
   CK(cudaMemsetAsync(c->r, 0, sizeof(double) * c->N, c->st));
   double best_us = 0.0;
   int best = 0;
-  for (int s = 0; s < nsaddle; ++s) {
-    c->saddle_shape = s;
+  const bool small = c->dim == 2 && c->lv[c->L - 1].Nc <= kTileSmallCells;
+  for (int s = 0; s < nsaddle + small; ++s) {
+    c->saddle_shape = s < nsaddle ? s : kTileSmall2D;
     double us;
     CKS(time_launches(c, [&]() -> cudaError_t {
       return saddle(c, TILE_APPLY, c->r, c->w, nullptr) == GS_OK ? cudaSuccess : cudaErrorUnknown; }, 3, &us));
-    if (s == 0 || us < 0.98 * best_us) { best_us = us; best = s; }
+    if (s == 0 || us < 0.98 * best_us) { best_us = us; best = c->saddle_shape; }
   }
   c->saddle_shape = best;
   return GS_OK;
@@ -3082,7 +3084,7 @@ gs_status gs_get_info(const gs_ctx* c, gs_info* out) {
   out->schur_cc = c->cc ? 1 : 0;
   out->pressure_coarse_free = c->nfp;
   for (int l = 0; l < c->L && l < 16; ++l) out->plambda_max[l] = c->lv[l].plam_hi;
-  static const int rows[kTileShapes2D] = {16, 17, 8, 0};
+  static const int rows[kTileSmall2D + 1] = {16, 17, 8, 0, 8};
   for (int l = 0; l < c->L && l < 16; ++l)
     out->tile_rows[l] = c->dim == 2 ? rows[c->lv[l].shape] : tile3d_depth(c->lv[l].shape);
   out->saddle_tile_rows = c->dim == 2 ? rows[c->saddle_shape] : tile3d_depth(c->saddle_shape);

@@ -43,11 +43,15 @@ struct TileArgs {
   T ihz;                // 1 / h_z (3D)
   int tiles[3];
   int shape;      // 2D velocity-block variant (0 / 1 / 2: tiles of 16 / 17 / 8 rows of evaluated cells,
-                  // 3: the strip kernel of gs_strip2d.cuh; other operator blocks: 3 -> tiles of 8);
+                  // 3: the strip kernel of gs_strip2d.cuh; other operator blocks: 3 -> tiles of 8;
+                  // 4: tiles of 8 x 8 evaluated cells);
                   // 3D: 0 / 1 -> segments of the length the launcher chooses / at most 4 evaluated layers
 };
 constexpr int kTileShapes2D = 4;   // velocity-block variants the autotuner times
 constexpr int kTileHeights2D = 3;  // tile variants of the full saddle operator
+constexpr int kTileSmall2D = 4;    // 8 x 8 tiles: timed too on meshes of at most kTileSmallCells cells, which
+                                   // 32-wide tiles of 465 owned cells cannot spread over twice the 152 SMs
+constexpr long long kTileSmallCells = 1LL << 17;
 // 3D march kernel (TileArgs::shape): 0 -> segment length by size, 1 -> at most 4 evaluated cell layers;
 // every node sums its cells in the same order, so the choice does not change any result
 constexpr int kTileShapes3D = 2;

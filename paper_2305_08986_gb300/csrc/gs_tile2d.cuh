@@ -14,7 +14,7 @@
 //      memory;
 //   3. each owned node sums the <= 4 cell results that touch it, in a fixed order (so the
 //      result does not depend on scheduling), and applies the mode's epilogue.
-// Threads form a 32 x 8 grid.  In phases 1 and 3 thread (tx, ty) handles node columns 2 tx and
+// Threads form an E0 x 8 grid (E0 = 32 or 8).  In phases 1 and 3 thread (tx, ty) handles node columns 2 tx and
 // 2 tx + 1 and node rows ty + 8 r, so the parity of its nodes is fixed (no per-node index
 // arithmetic, uniform branches within a warp) and it consumes the epilogue operands it staged.
 #pragma once
@@ -24,14 +24,14 @@
 namespace gs {
 
 namespace tile2d {
-constexpr int NT = 256;      // threads per CTA: 32 x 8
-constexpr int TY = NT / 32;  // 8
+constexpr int TY = 8;  // thread rows per CTA
 
-// Tile shape: 32 x EY evaluated cells (EY = 16 by default; the per-level autotuner may pick
-// another compiled height, see launch_tile2d).
-template <int EY>
+// Tile shape: EX x EY evaluated cells, EX x 8 threads (32 x 16 by default; the per-level autotuner may
+// pick another compiled shape, see launch_tile2d).
+template <int EX, int EY>
 struct Shape2 {
-  static constexpr int E0 = 32, E1 = EY;                  // evaluated cells per tile
+  static constexpr int NT = EX * TY;                      // threads per CTA
+  static constexpr int E0 = EX, E1 = EY;                  // evaluated cells per tile
   static constexpr int TO0 = E0 - 1, TO1 = E1 - 1;        // owned cells per tile
   static constexpr int NCELL = E0 * E1;
   static constexpr int IN0 = 2 * E0 + 1, IN1 = 2 * E1 + 1;  // velocity input node tile
@@ -46,21 +46,21 @@ struct Shape2 {
   static constexpr int CROWS = (E1 + TY - 1) / TY;        // evaluated cell rows per thread
 };
 
-#define GS_SHAPE2_NAMES(EY)                                                                    \
-  using S2__ = Shape2<EY>;                                                                     \
+#define GS_SHAPE2_NAMES(SH)                                                                    \
+  using S2__ = SH;                                                                             \
   constexpr int E0 = S2__::E0, E1 = S2__::E1, TO0 = S2__::TO0, TO1 = S2__::TO1;               \
   constexpr int NCELL = S2__::NCELL, IN0 = S2__::IN0, IN1 = S2__::IN1, NIN = S2__::NIN;        \
   constexpr int PI0 = S2__::PI0, PI1 = S2__::PI1, VP0 = S2__::VP0, VP1 = S2__::VP1;           \
   constexpr int OWN = S2__::OWN, PP0 = S2__::PP0, PP1 = S2__::PP1, POWN = S2__::POWN;         \
-  constexpr int ROWS = S2__::ROWS, IROWS = S2__::IROWS, CROWS = S2__::CROWS;                  \
+  constexpr int ROWS = S2__::ROWS, IROWS = S2__::IROWS, CROWS = S2__::CROWS, NT = S2__::NT;   \
   (void)E0; (void)E1; (void)TO0; (void)TO1; (void)NCELL; (void)IN0; (void)IN1; (void)NIN;      \
   (void)PI0; (void)PI1; (void)VP0; (void)VP1; (void)OWN; (void)PP0; (void)PP1; (void)POWN;    \
-  (void)ROWS; (void)IROWS; (void)CROWS
+  (void)ROWS; (void)IROWS; (void)CROWS; (void)NT
 
-template <int EY, int MODE, bool NEED_U, bool WBT, bool WU, bool WB, int CONV = 0>
+template <class S2, int MODE, bool NEED_U, bool WBT, bool WU, bool WB, int CONV = 0>
 struct Smem2 {
-  static constexpr int NIN = Shape2<EY>::NIN, PI0 = Shape2<EY>::PI0, PI1 = Shape2<EY>::PI1;
-  static constexpr int NCELL = Shape2<EY>::NCELL, OWN = Shape2<EY>::OWN, POWN = Shape2<EY>::POWN;
+  static constexpr int NIN = S2::NIN, PI0 = S2::PI0, PI1 = S2::PI1;
+  static constexpr int NCELL = S2::NCELL, OWN = S2::OWN, POWN = S2::POWN;
   static constexpr int SX = NEED_U ? 2 * NIN : 0;
   static constexpr int SP = WBT ? PI0 * PI1 : 0;
   static constexpr int RU = WU ? 18 * NCELL : 0;
@@ -95,9 +95,9 @@ __device__ __forceinline__ int owned_ext(int cs, int TO, int n, int mult) {
 // Sum of the cell results touching owned node (i0, i1), with the node's local positions fixed by
 // its parities (even: local 0 in the next cell and local 2 in the previous one; odd: local 1).
 // Evaluated cell index = cell + 1 - cs; indices beyond the evaluated range lie outside the mesh.
-template <typename T, int EY, bool XODD, bool YODD>
+template <typename T, class S2, bool XODD, bool YODD>
 __device__ __forceinline__ void gather2(const T* ru, int i0, int i1, T& s0, T& s1) {
-  GS_SHAPE2_NAMES(EY);
+  GS_SHAPE2_NAMES(S2);
   s0 = T(0);
   s1 = T(0);
   const int ey0 = YODD ? (i1 + 1) >> 1 : (i1 >> 1) + 1;
@@ -119,12 +119,12 @@ __device__ __forceinline__ void gather2(const T* ru, int i0, int i1, T& s0, T& s
     }
   }
 }
-template <typename T, int EY, int MODE, bool WA, bool WBT, bool WB, int CONV = 0>
+template <typename T, class S2, int MODE, bool WA, bool WBT, bool WB, int CONV = 0>
 __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
-  GS_SHAPE2_NAMES(EY);
+  GS_SHAPE2_NAMES(S2);
   constexpr bool NEED_U = WA || WB;
   constexpr bool WU = WA || WBT;
-  using SM = Smem2<EY, MODE, NEED_U, WBT, WU, WB, CONV>;
+  using SM = Smem2<S2, MODE, NEED_U, WBT, WU, WB, CONV>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sx = reinterpret_cast<T*>(smem_raw);
   T* sp = sx + SM::SX;
@@ -144,7 +144,7 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
   const int cs0 = t0 * TO0, cs1 = t1 * TO1;
   const long long Nv = g.Nv;
   const int tid = threadIdx.x;
-  const int tx = tid & 31, ty = tid >> 5;
+  const int tx = tid % E0, ty = tid / E0;
   const int ve0 = owned_ext(cs0, TO0, g.n[0], 2), ve1 = owned_ext(cs1, TO1, g.n[1], 2);
   const int pe0 = owned_ext(cs0, TO0, g.n[0], 1), pe1 = owned_ext(cs1, TO1, g.n[1], 1);
   const bool vmasked = !raw && g.vmask != nullptr;
@@ -160,7 +160,7 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
       const bool rowok = iy < IN1 && J >= 0 && J < g.nv[1];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const int ix = tx + 32 * q;
+        const int ix = tx + E0 * q;
         mk[3 * r + q] = 0;
         if (iy < IN1 && ix < IN0) {
           const int I = I0 + ix;
@@ -225,7 +225,7 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
       const int iy = ty + TY * r;
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const int ix = tx + 32 * q;
+        const int ix = tx + E0 * q;
         if (iy < IN1 && ix < IN0) scon[ix + IN0 * iy] = mk[3 * r + q];
       }
     }
@@ -238,7 +238,7 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
       const int iy = ty + TY * r;
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        const int ix = tx + 32 * q;
+        const int ix = tx + E0 * q;
         if (iy < IN1 && ix < IN0 && mk[3 * r + q]) {
           sx[ix + IN0 * iy] = T(0);
           sx[NIN + ix + IN0 * iy] = T(0);
@@ -248,7 +248,7 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
   }
   __syncthreads();
 
-  // ---- phase 2: evaluate cells; thread (tx, ty) -> cells (tx, ty) and (tx, ty + 8) ----
+  // ---- phase 2: evaluate cells; thread (tx, ty) -> cells (tx, ty + 8 k) ----
 #pragma unroll 1
   for (int k = 0; k < CROWS; ++k) {
     const int e0 = tx, e1 = ty + TY * k;
@@ -327,11 +327,11 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
         if (i0 >= ve0) continue;
         T s0, s1;
         if (ty & 1) {
-          if (q) gather2<T, EY, true, true>(ru, i0, i1, s0, s1);
-          else gather2<T, EY, false, true>(ru, i0, i1, s0, s1);
+          if (q) gather2<T, S2, true, true>(ru, i0, i1, s0, s1);
+          else gather2<T, S2, false, true>(ru, i0, i1, s0, s1);
         } else {
-          if (q) gather2<T, EY, true, false>(ru, i0, i1, s0, s1);
-          else gather2<T, EY, false, false>(ru, i0, i1, s0, s1);
+          if (q) gather2<T, S2, true, false>(ru, i0, i1, s0, s1);
+          else gather2<T, S2, false, false>(ru, i0, i1, s0, s1);
         }
         const long long node = (2 * cs0 + i0) + (long long)g.nv[0] * (2 * cs1 + i1);
         const int sidx = (i0 + 2) + IN0 * (i1 + 2);  // the node in the staged input tile
@@ -383,83 +383,80 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
   }
 }
 
-template <typename T, int EY, int MODE, bool WA, bool WBT, bool WB, int CONV = 0>
+template <typename T, class S2, int MODE, bool WA, bool WBT, bool WB, int CONV = 0>
 struct Tile2dK {
   using Args = TileArgs<T>;
   // FP64 with B^T (the saddle operator, FP64-pipe-bound): 3 CTAs per SM (76 registers).  1280 x 224: 138 us
   // with the cells in Legendre modes (~180 FP64 operations per cell), 260 us in 3 x 3 sweeps (~400); the
   // FP32 variants stay at 2
-  static constexpr int THREADS = NT, MINB = CONV ? 1 : (sizeof(T) == 8 && WBT ? 3 : 2);
+  static constexpr int THREADS = S2::NT, MINB = CONV ? 1 : (S2::E0 == 8 ? 8 : (sizeof(T) == 8 && WBT ? 3 : 2));
   static __device__ __forceinline__ void body(const Args& a, int blk, int) {
-    tile2d_body<T, EY, MODE, WA, WBT, WB, CONV>(a, blk);
+    tile2d_body<T, S2, MODE, WA, WBT, WB, CONV>(a, blk);
   }
 };
 
-template <typename T, int EY, int MODE, bool WA, bool WBT, bool WB, int CONV = 0>
+template <typename T, class S2, int MODE, bool WA, bool WBT, bool WB, int CONV = 0>
 cudaError_t launch2(TileArgs<T> a, cudaStream_t st) {
-  using S2 = Shape2<EY>;
-  using SM = Smem2<EY, MODE, WA || WB, WBT, WA || WBT, WB, CONV>;
+  using SM = Smem2<S2, MODE, WA || WB, WBT, WA || WBT, WB, CONV>;
   a.tiles[0] = (a.g.n[0] + S2::TO0 - 1) / S2::TO0;
   a.tiles[1] = (a.g.n[1] + S2::TO1 - 1) / S2::TO1;
   a.tiles[2] = 1;
   const size_t smem = sizeof(T) * SM::TOTAL + SM::FLAGS;
-  return submit<Tile2dK<T, EY, MODE, WA, WBT, WB, CONV>>(a, (long long)a.tiles[0] * a.tiles[1], smem, st);
+  return submit<Tile2dK<T, S2, MODE, WA, WBT, WB, CONV>>(a, (long long)a.tiles[0] * a.tiles[1], smem, st);
 }
 
 // Velocity block and saddle operator with the corrector-stage terms (cell_conv2): conv = 1 adds
 // rho (C + S), conv = 2 the symmetric part rho (S + (C + C^T) / 2) (velocity block only).
-template <typename T, int EY>
+template <typename T, class S2>
 cudaError_t launch_conv_shape(int mode, int ops, const TileArgs<T>& a, cudaStream_t st) {
   if (ops == OPS_A) {
     if (a.conv == 2) {
-      if (mode == TILE_APPLY) return launch2<T, EY, TILE_APPLY, true, false, false, 2>(a, st);
+      if (mode == TILE_APPLY) return launch2<T, S2, TILE_APPLY, true, false, false, 2>(a, st);
       return cudaErrorInvalidValue;
     }
-    if (mode == TILE_APPLY) return launch2<T, EY, TILE_APPLY, true, false, false, 1>(a, st);
-    if (mode == TILE_RESID) return launch2<T, EY, TILE_RESID, true, false, false, 1>(a, st);
-    return launch2<T, EY, TILE_CHEB, true, false, false, 1>(a, st);
+    if (mode == TILE_APPLY) return launch2<T, S2, TILE_APPLY, true, false, false, 1>(a, st);
+    if (mode == TILE_RESID) return launch2<T, S2, TILE_RESID, true, false, false, 1>(a, st);
+    return launch2<T, S2, TILE_CHEB, true, false, false, 1>(a, st);
   }
   if (ops == (OPS_A | OPS_BT | OPS_B) && a.conv == 1) {
-    return mode == TILE_APPLY ? launch2<T, EY, TILE_APPLY, true, true, true, 1>(a, st)
-                              : launch2<T, EY, TILE_RESID, true, true, true, 1>(a, st);
+    return mode == TILE_APPLY ? launch2<T, S2, TILE_APPLY, true, true, true, 1>(a, st)
+                              : launch2<T, S2, TILE_RESID, true, true, true, 1>(a, st);
   }
   return cudaErrorInvalidValue;
 }
 
-// Launch one tile height.  FULL: every mode / operator combination is compiled; otherwise only
-// the velocity-block modes the multigrid uses on every level (apply, residual, Chebyshev).
-template <typename T, int EY, bool FULL>
+// Launch one tile shape.
+template <typename T, class S2>
 cudaError_t launch_shape(int mode, int ops, const TileArgs<T>& a, cudaStream_t st) {
   if (ops == OPS_A) {
-    if (mode == TILE_APPLY) return launch2<T, EY, TILE_APPLY, true, false, false>(a, st);
-    if (mode == TILE_RESID) return launch2<T, EY, TILE_RESID, true, false, false>(a, st);
-    return launch2<T, EY, TILE_CHEB, true, false, false>(a, st);
+    if (mode == TILE_APPLY) return launch2<T, S2, TILE_APPLY, true, false, false>(a, st);
+    if (mode == TILE_RESID) return launch2<T, S2, TILE_RESID, true, false, false>(a, st);
+    return launch2<T, S2, TILE_CHEB, true, false, false>(a, st);
   }
-  if constexpr (FULL) {
-    if (mode == TILE_CHEB) return cudaErrorInvalidValue;
-    const bool ap = mode == TILE_APPLY;
-    switch (ops) {
-      case OPS_BT:
-        return ap ? launch2<T, EY, TILE_APPLY, false, true, false>(a, st) : launch2<T, EY, TILE_RESID, false, true, false>(a, st);
-      case OPS_B:
-        return ap ? launch2<T, EY, TILE_APPLY, false, false, true>(a, st) : launch2<T, EY, TILE_RESID, false, false, true>(a, st);
-      case OPS_A | OPS_BT | OPS_B:
-        return ap ? launch2<T, EY, TILE_APPLY, true, true, true>(a, st) : launch2<T, EY, TILE_RESID, true, true, true>(a, st);
-      default:
-        return cudaErrorInvalidValue;
-    }
+  if (mode == TILE_CHEB) return cudaErrorInvalidValue;
+  const bool ap = mode == TILE_APPLY;
+  switch (ops) {
+    case OPS_BT:
+      return ap ? launch2<T, S2, TILE_APPLY, false, true, false>(a, st) : launch2<T, S2, TILE_RESID, false, true, false>(a, st);
+    case OPS_B:
+      return ap ? launch2<T, S2, TILE_APPLY, false, false, true>(a, st) : launch2<T, S2, TILE_RESID, false, false, true>(a, st);
+    case OPS_A | OPS_BT | OPS_B:
+      return ap ? launch2<T, S2, TILE_APPLY, true, true, true>(a, st) : launch2<T, S2, TILE_RESID, true, true, true>(a, st);
+    default:
+      return cudaErrorInvalidValue;
   }
-  return cudaErrorNotSupported;
 }
 
 }  // namespace tile2d
 
-// per-height launchers (one translation unit each, compiled in parallel)
+// per-shape launchers (one translation unit each, compiled in parallel)
 template <typename T>
 cudaError_t launch_tile2d_e16(int mode, int ops, const TileArgs<T>& a, cudaStream_t st);
 template <typename T>
 cudaError_t launch_tile2d_e17(int mode, int ops, const TileArgs<T>& a, cudaStream_t st);
 template <typename T>
 cudaError_t launch_tile2d_e8(int mode, int ops, const TileArgs<T>& a, cudaStream_t st);
+template <typename T>
+cudaError_t launch_tile2d_x8(int mode, int ops, const TileArgs<T>& a, cudaStream_t st);
 
 }  // namespace gs

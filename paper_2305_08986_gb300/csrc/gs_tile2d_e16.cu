@@ -5,7 +5,7 @@ namespace gs {
 
 template <typename T>
 cudaError_t launch_tile2d_e16(int mode, int ops, const TileArgs<T>& a, cudaStream_t st) {
-  return tile2d::launch_shape<T, 16, true>(mode, ops, a, st);
+  return tile2d::launch_shape<T, tile2d::Shape2<32, 16>>(mode, ops, a, st);
 }
 template cudaError_t launch_tile2d_e16<float>(int, int, const TileArgs<float>&, cudaStream_t);
 template cudaError_t launch_tile2d_e16<double>(int, int, const TileArgs<double>&, cudaStream_t);
@@ -16,7 +16,7 @@ namespace gs {
 
 // Variant per launch: TileArgs::shape 0 -> tiles of 16 rows of evaluated cells, 1 -> 17, 2 -> 8,
 // 3 -> the strip kernel for the velocity block (gs_strip2d.cu; tiles of 8 rows for the other
-// blocks).  The result does not depend on the variant: every node sums its cell contributions in
+// blocks), 4 -> tiles of 8 x 8 evaluated cells (coarse levels and small meshes).  The result does not depend on the variant: every node sums its cell contributions in
 // the same fixed order.
 template <typename T>
 cudaError_t launch_tile2d(int mode, int ops, TileArgs<T> a, cudaStream_t st) {
@@ -28,6 +28,7 @@ cudaError_t launch_tile2d(int mode, int ops, TileArgs<T> a, cudaStream_t st) {
   if (a.shape == 3 && ops == OPS_A && 2 * a.g.Nv < (1LL << 31)) return launch_strip2d<T>(mode, a, st);
   if (a.shape == 1) return launch_tile2d_e17<T>(mode, ops, a, st);
   if (a.shape == 2 || a.shape == 3) return launch_tile2d_e8<T>(mode, ops, a, st);
+  if (a.shape == 4) return launch_tile2d_x8<T>(mode, ops, a, st);
   return launch_tile2d_e16<T>(mode, ops, a, st);
 }
 template cudaError_t launch_tile2d<float>(int, int, TileArgs<float>, cudaStream_t);

@@ -5,7 +5,7 @@ namespace gs {
 
 template <typename T>
 cudaError_t launch_tile2d_e17(int mode, int ops, const TileArgs<T>& a, cudaStream_t st) {
-  return tile2d::launch_shape<T, 17, true>(mode, ops, a, st);
+  return tile2d::launch_shape<T, tile2d::Shape2<32, 17>>(mode, ops, a, st);
 }
 template cudaError_t launch_tile2d_e17<float>(int, int, const TileArgs<float>&, cudaStream_t);
 template cudaError_t launch_tile2d_e17<double>(int, int, const TileArgs<double>&, cudaStream_t);
