@@ -1524,7 +1524,8 @@ gs_status pcheb(gs_ctx* c, int l, const T* b, bool zero_init, bool started = fal
   return GS_OK;
 }
 
-// V-cycle for the pressure Laplacian: input lv.pb, output lv.pxA
+// V-cycle for the pressure Laplacian: input lv.pb, output lv.pxA.  General smoother; pvcycle_deg2 below
+// runs the default one in two launches per level.
 template <typename T>
 gs_status pvcycle(gs_ctx* c, int l, bool started = false) {
   const LevelTag tag__(c, l);
@@ -1553,11 +1554,42 @@ gs_status pvcycle(gs_ctx* c, int l, bool started = false) {
   return GS_OK;
 }
 
+// The same cycle for one smoothing step of degree 2 on level l >= 1, right-hand side b
+template <typename T>
+gs_status pvcycle_deg2(gs_ctx* c, int l, const T* b) {
+  const LevelTag tag__(c, l);
+  Level& lv = c->lv[l];
+  Level& cl = c->lv[l - 1];
+  const PLapArgs<T> p = plap_args<T>(lv);
+  const double hi = lv.plam_hi, lo = hi / 15.0;
+  const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo), sigma = theta / delta, rho = 1.0 / sigma;
+  const double rn = 1.0 / (2.0 * sigma - rho);
+  Q1CycleArgs<T> a{};
+  a.gf = lv.g; a.gc = cl.g; a.w = p.w; a.mf = lv.pcmask; a.mc = cl.pcmask;
+  for (int i = 0; i < 3; ++i) a.kc[i] = p.kc[i];
+  a.b = b; a.dinv = (const T*)lv.pdinv; a.x = (T*)lv.pxA; a.bc = (T*)cl.pb;
+  a.inv_theta = (T)(1.0 / theta); a.c1 = (T)(rn * rho); a.c2 = (T)(2.0 * rn / delta);
+  const bool start = l == 1 && c->opt.coarse_mode == 1;  // level 0 is smoothed from zero
+  if (start) {
+    a.sd = (T*)cl.pd; a.sx = (T*)cl.pxA; a.sdinv = (const T*)cl.pdinv; a.s_inv_theta = (T)cheb_inv_theta(cl.plam_hi);
+  }
+  KL(K_SCHUR, launch_q1cycle<T>(0, a, c->st));
+  if (l > 1)
+    CKS(pvcycle_deg2<T>(c, l - 1, (const T*)cl.pb));
+  else
+    CKS(pvcycle<T>(c, 0, start));
+  a.e = (const T*)cl.pxA; a.xout = (T*)lv.pxB;
+  KL(K_SCHUR, launch_q1cycle<T>(1, a, c->st));
+  std::swap(lv.pxA, lv.pxB);
+  return GS_OK;
+}
+
 // Cahouet-Chabard term K_p^{-1} r ~ one pressure V-cycle, constrained entries zero; result in
 // the finest level's pxA
 template <typename T>
 gs_status plap_inverse(gs_ctx* c, const T* r) {
   Level& F = c->lv[c->L - 1];
+  if (c->L > 1 && c->opt.smooth_steps == 1 && c->opt.plap_degree == 2) return pvcycle_deg2<T>(c, c->L - 1, r);
   KL(K_VEC, launch_mask_copy<T>(r, F.pcmask, (T*)F.pb, F.Np, c->st));
   CKS(pvcycle<T>(c, c->L - 1));
   return GS_OK;

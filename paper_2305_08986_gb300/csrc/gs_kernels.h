@@ -172,6 +172,26 @@ struct Q1Args {
 };
 template <typename T>
 cudaError_t launch_q1tile(int op, int mode, const Q1Args<T>& a, cudaStream_t st);
+// One half of a level in the pressure-Laplacian V-cycle (gs_q1cycle.cu), smoother degree 2, one smoothing step:
+// up = 0: x <- smoother from zero on b, bc <- R (b - K x); up = 1: xout <- smoother from x + P e.
+template <typename T>
+struct Q1CycleArgs {
+  Geom gf, gc;
+  T kc[3];
+  const T* w;               // per-cell weight (NULL: 1)
+  const uint8_t *mf, *mc;   // masks of the level and of the coarse one
+  const T* b;               // right-hand side (masked entries are taken as zero)
+  const T* dinv;
+  T* x;                     // the level's iterate (down: output, up: input)
+  T* bc;                    // down: coarse right-hand side
+  T *sd, *sx;               // down: start of the coarse smoother, d = x = sdinv * bc * s_inv_theta (NULL: none)
+  const T* sdinv;
+  const T* e;               // up: coarse correction
+  T* xout;                  // up: result (must not alias x)
+  T inv_theta, c1, c2, s_inv_theta;
+};
+template <typename T>
+cudaError_t launch_q1cycle(int up, const Q1CycleArgs<T>& a, cudaStream_t st);
 // out[i] = mask[i] ? 0 : in[i]   (may run in place)
 template <typename T>
 cudaError_t launch_mask_copy(const T* in, const uint8_t* mask, T* out, long long n, cudaStream_t st);
