@@ -131,7 +131,8 @@ typedef struct {            /* zero-initialised = defaults */
                                   1 / 2 / 3 -> always the 32 x 16 / 32 x 17 / 32 x 8 tile; 4 -> always
                                   the strip kernel (the FP64 saddle operator then uses 32 x 8 tiles);
                                   5 -> by size, the strip kernel on levels of at least 32,768 cells
-                                  and 32 x 8 tiles below (no timing at gs_create).
+                                  and 32 x 8 tiles below (no timing at gs_create); 6 -> always
+                                  8 x 8 tiles.
                                3D meshes: 0 -> time cell-layer segments of the length chosen by size
                                   and of at most 4 evaluated layers per level and keep the faster
                                   (default); 2 -> always at most 4 layers; any other value -> always

@@ -268,7 +268,7 @@ gs_options normalize_opts(const gs_options* o) {
   r.plap_degree = opt_or(r.plap_degree, 2);
   // 0 (default) and 1: IEEE FP64 basis; 2: double-float basis (stored internally as 0 / 1 = double-float / FP64)
   r.krylov_fp64 = r.krylov_fp64 == 2 ? 0 : 1;
-  r.tile_autotune = (r.tile_autotune >= 1 && r.tile_autotune <= 5) ? r.tile_autotune : 0;
+  r.tile_autotune = (r.tile_autotune >= 1 && r.tile_autotune <= 6) ? r.tile_autotune : 0;
   r.corrector = r.corrector == 1 ? 1 : 0;
   r.deflate = r.deflate == 1 ? 1 : 0;
   r.precond_kind = r.precond_kind == 1 ? 1 : 0;
@@ -1390,6 +1390,9 @@ gs_status setup(gs_ctx* c) {
     // size rule: the strip kernel where a level has enough cells to fill the GPU, 32 x 8 tiles below
     for (int l = 0; l < c->L; ++l) c->lv[l].shape = c->lv[l].Nc >= 32768 ? 3 : 2;
     c->saddle_shape = 2;
+  } else if (c->dim == 2 && c->opt.tile_autotune == 6) {
+    for (int l = 0; l < c->L; ++l) c->lv[l].shape = kTileSmall2D;
+    c->saddle_shape = kTileSmall2D;
   } else if (c->dim == 2) {
     for (int l = 0; l < c->L; ++l) c->lv[l].shape = c->opt.tile_autotune - 1;
     c->saddle_shape = std::min(c->opt.tile_autotune - 1, kTileHeights2D - 1);
@@ -1402,9 +1405,11 @@ gs_status setup(gs_ctx* c) {
 double cheb_inv_theta(double hi) { return 1.0 / (0.5 * (hi + hi / 15.0)); }
 
 // started: the first step from zero (d = x = dinv b / theta) was already done by the restriction
-// that produced b (launch_restrict with a Chebyshev start)
+// that produced b (launch_restrict with a Chebyshev start).  x0 (zero_init false): the start, instead of
+// lv.xA.  out: where the last step leaves the result, instead of lv.xA; it overlaps neither b nor x0.
 template <typename T>
-gs_status cheb(gs_ctx* c, int l, const T* b, bool zero_init, bool started = false) {
+gs_status cheb(gs_ctx* c, int l, const T* b, bool zero_init, bool started = false, const T* x0 = nullptr,
+               T* out = nullptr) {
   const LevelTag tag__(c, l);
   Level& lv = c->lv[l];
   const double hi = lv.lam_hi, lo = hi / 15.0;
@@ -1412,42 +1417,58 @@ gs_status cheb(gs_ctx* c, int l, const T* b, bool zero_init, bool started = fals
   const int k = c->opt.cheb_degree;
   T* dinv = (T*)lv.dinv;
   T* d = (T*)lv.d;
+  const T* cur = x0 ? x0 : (const T*)lv.xA;
+  auto step = [&](T c1, T c2, int use_d, bool last) -> gs_status {
+    T* const to = last && out ? out : (T*)lv.xB;
+    TileArgs<T> a = tile_args<T>(lv);
+    a.xu = cur; a.bu = b; a.d = d; a.dinv = dinv; a.xout = to;
+    a.c1 = c1; a.c2 = c2; a.use_d = use_d;
+    KL(K_CHEB, launch_tile<T>(c->dim, TILE_CHEB, OPS_A, a, c->st));
+    if (to != out) std::swap(lv.xA, lv.xB);
+    cur = to;
+    return GS_OK;
+  };
   if (zero_init) {
     if (!started) KL(K_VEC, launch_cheb_init0<T>(b, dinv, (T)(1.0 / theta), d, (T*)lv.xA, lv.nu, c->st));
+    cur = (const T*)lv.xA;
   } else {
-    TileArgs<T> a = tile_args<T>(lv);
-    a.xu = (const T*)lv.xA; a.bu = b; a.d = d; a.dinv = dinv; a.xout = (T*)lv.xB;
-    a.c1 = 0; a.c2 = (T)(1.0 / theta); a.use_d = 0;
-    KL(K_CHEB, launch_tile<T>(c->dim, TILE_CHEB, OPS_A, a, c->st));
-    std::swap(lv.xA, lv.xB);
+    CKS(step((T)0, (T)(1.0 / theta), 0, k <= 1));
   }
   double rho = 1.0 / sigma;
   for (int t = 1; t < k; ++t) {
     const double rn = 1.0 / (2.0 * sigma - rho);
-    TileArgs<T> a = tile_args<T>(lv);
-    a.xu = (const T*)lv.xA; a.bu = b; a.d = d; a.dinv = dinv; a.xout = (T*)lv.xB;
-    a.c1 = (T)(rn * rho); a.c2 = (T)(2.0 * rn / delta); a.use_d = 1;
-    KL(K_CHEB, launch_tile<T>(c->dim, TILE_CHEB, OPS_A, a, c->st));
-    std::swap(lv.xA, lv.xB);
+    CKS(step((T)(rn * rho), (T)(2.0 * rn / delta), 1, t == k - 1));
     rho = rn;
   }
+  if (out && cur != out)  // degree 1 from zero: no step
+    CK(cudaMemcpyAsync(out, cur, sizeof(T) * lv.nu, cudaMemcpyDeviceToDevice, c->st));
   return GS_OK;
 }
 
-// V-cycle on level l: input lv.b, output lv.xA (started: see cheb)
+// Whether the kernels may work on the caller's vectors in place of copies: element-aligned, and y apart
+// from the inputs.
 template <typename T>
-gs_status vcycle(gs_ctx* c, int l, bool started = false) {
+bool direct(long long n, const T* y, const T* x, const T* aux = nullptr) {
+  const uintptr_t Y = (uintptr_t)y, bytes = sizeof(T) * (uintptr_t)n;
+  auto apart = [&](const T* p) { return Y + bytes <= (uintptr_t)p || (uintptr_t)p + bytes <= Y; };
+  return (Y | (uintptr_t)x | (uintptr_t)aux) % sizeof(T) == 0 && apart(x) && (!aux || apart(aux));
+}
+
+// V-cycle on level l: input b (NULL: lv.b), output out (NULL: lv.xA; not on level 0) (started: see cheb)
+template <typename T>
+gs_status vcycle(gs_ctx* c, int l, bool started = false, const T* b = nullptr, T* out = nullptr) {
   const LevelTag tag__(c, l);
   Level& lv = c->lv[l];
+  if (!b) b = (const T*)lv.b;
   if (l == 0) {
-    if (c->opt.coarse_mode == 1) return cheb<T>(c, 0, (const T*)lv.b, true, started);
-    KL(K_COARSE, launch_coarse_solve<T>(c->Ainv, c->cfree, c->nf, (const T*)lv.b, (T*)lv.xA, lv.nu, c->ctmp, c->st));
+    if (c->opt.coarse_mode == 1) return cheb<T>(c, 0, b, true, started);
+    KL(K_COARSE, launch_coarse_solve<T>(c->Ainv, c->cfree, c->nf, b, (T*)lv.xA, lv.nu, c->ctmp, c->st));
     return GS_OK;
   }
-  for (int s = 0; s < c->opt.smooth_steps; ++s) CKS(cheb<T>(c, l, (const T*)lv.b, s == 0, s == 0 && started));
+  for (int s = 0; s < c->opt.smooth_steps; ++s) CKS(cheb<T>(c, l, b, s == 0, s == 0 && started));
   {
     TileArgs<T> a = tile_args<T>(lv);
-    a.xu = (const T*)lv.xA; a.bu = (const T*)lv.b; a.yu = (T*)lv.d;
+    a.xu = (const T*)lv.xA; a.bu = b; a.yu = (T*)lv.d;
     KL(K_RESID, launch_tile<T>(c->dim, TILE_RESID, OPS_A, a, c->st));
   }
   // rigid-body deflation on the finest level: y = E^-1 Z^T r, added after the coarse correction
@@ -1467,7 +1488,8 @@ gs_status vcycle(gs_ctx* c, int l, bool started = false) {
   CKS(vcycle<T>(c, l - 1, start));
   KL(K_TRANSFER, launch_prolong_add<T>(lv.g, cl.g, (const T*)cl.xA, (T*)lv.xA, c->st));
   if (defl) KL(K_VEC, launch_defl_add<T>(c->defl, c->d_y, (T*)lv.xA, c->st));
-  for (int s = 0; s < c->opt.smooth_steps; ++s) CKS(cheb<T>(c, l, (const T*)lv.b, false));
+  for (int s = 0; s < c->opt.smooth_steps; ++s)
+    CKS(cheb<T>(c, l, b, false, false, nullptr, s == c->opt.smooth_steps - 1 ? out : nullptr));
   return GS_OK;
 }
 
@@ -2127,6 +2149,8 @@ gs_status apply_level_T(gs_ctx* c, int l, gs_op op, const void* xv, void* yv, co
     case GS_OP_SMOOTH: {
       if (!mgprec || (l == 0 && c->opt.coarse_mode != 1))
         return fail(GS_EINVAL, "smoother: level >= 1 (or level 0 with coarse_mode 1), MG precision");
+      if (c->opt.smooth_steps == 1 && direct(lv.nu, (const T*)y, x, aux))
+        return cheb<T>(c, l, x, !aux, false, aux, y);
       if (aux) CK(cudaMemcpyAsync(lv.xA, aux, sizeof(T) * lv.nu, cudaMemcpyDeviceToDevice, c->st));
       CK(cudaMemcpyAsync(lv.b, x, sizeof(T) * lv.nu, cudaMemcpyDeviceToDevice, c->st));
       for (int s = 0; s < c->opt.smooth_steps; ++s) CKS(cheb<T>(c, l, (const T*)lv.b, s == 0 && !aux));
@@ -2763,6 +2787,8 @@ gs_status gs_vcycle(gs_ctx* c, const double* r, double* z) {
     CKS(vcycle<float>(c, c->L - 1));
     CK(launch_cast<float, double>((const float*)F.xA, z, F.nu, 1.0, c->st));
   } else {
+    if (c->L > 1 && c->opt.smooth_steps > 0 && direct(F.nu, (const double*)z, r))
+      return vcycle<double>(c, c->L - 1, false, r, z);
     CK(cudaMemcpyAsync(F.b, r, sizeof(double) * F.nu, cudaMemcpyDeviceToDevice, c->st));
     CKS(vcycle<double>(c, c->L - 1));
     CK(cudaMemcpyAsync(z, F.xA, sizeof(double) * F.nu, cudaMemcpyDeviceToDevice, c->st));
