@@ -114,8 +114,9 @@ __device__ __forceinline__ void gather2(const T* ru, int i0, int i1, T& s0, T& s
       if (ex >= E0) continue;
       const int e = ex + E0 * ey;
       const int li = la + 3 * lb;
-      s0 += ru[li * NCELL + e];
-      s1 += ru[(9 + li) * NCELL + e];
+      const T v0 = ru[li * NCELL + e], v1 = ru[(9 + li) * NCELL + e];
+      s0 = a + b == 0 ? v0 : s0 + v0;  // no addition to the zero: the FP64 pipe bounds the FP64 operators
+      s1 = a + b == 0 ? v1 : s1 + v1;
     }
   }
 }
