@@ -1,4 +1,4 @@
-// Node-gather kernels: diagonal of A, multigrid transfers, and the 1/eta-weighted pressure
+// Node-gather kernels: diagonal of A, pressure transfers, and the 1/eta-weighted pressure
 // mass (Schur approximation).  One thread per output node; every output is written once.
 #include "gs_cell.cuh"
 #include "gs_kernels.h"
@@ -83,30 +83,6 @@ cudaError_t launch_diagA(const Geom& g, const OpCoef<T>& c, const T* eta, const 
   return launched(cudaGetLastError());
 }
 
-// ---- transfers: P = Q2 interpolation of the coarse field at the fine nodes (Sec. 4, nested
-// meshes); R = P^T.  1D weights: fine 2C <- coarse C (1); fine 4c+1 <- (3/8, 3/4, -1/8) on
-// coarse (2c, 2c+1, 2c+2); fine 4c+3 <- (-1/8, 3/4, 3/8).  Constrained fine rows and
-// constrained coarse columns are removed. -----------------------------------------------------
-
-// weights of coarse node C seen from fine nodes, in five slots at offsets f - 2C = -3, -1, 0, 1, 3:
-// even C: (-1/8, 3/8, 1, 3/8, -1/8); odd C: (-, 3/4, 1, 3/4, -); ok marks the slots that exist
-// (inside the fine mesh, and the inner three for odd C).  Fixed slots, so the arrays stay in
-// registers when the loops over them are unrolled.  The weights and their pairwise products are
-// dyadic and exact in FP32, so they are kept in float (FP64 arithmetic is far slower on this GPU);
-// the results are the same bits.
-__device__ __forceinline__ void restrict_stencil(int C, int nvf, int (&fi)[5], float (&w)[5], bool (&ok)[5]) {
-  const bool odd = C & 1;
-  const int off[5] = {-3, -1, 0, 1, 3};
-#pragma unroll
-  for (int t = 0; t < 5; ++t) {
-    fi[t] = 2 * C + off[t];
-    ok[t] = fi[t] >= 0 && fi[t] < nvf && (!odd || (t >= 1 && t <= 3));
-  }
-  w[0] = w[4] = -0.125f;
-  w[1] = w[3] = odd ? 0.75f : 0.375f;
-  w[2] = 1.0f;
-}
-
 // Optional start of the coarse level's Chebyshev smoother from zero, fused into the restriction
 // that produces its right-hand side: d = x = dinv * rc * inv_theta (the same expression as the
 // separate start kernel, so the same bits).  d == NULL: restriction only.
@@ -117,147 +93,6 @@ struct ChebStart {
   T* d;
   T* x;
 };
-
-template <typename T>
-struct XferArgs {
-  Geom gf, gc;
-  const T* in;
-  T* out;
-  ChebStart<T> cs;
-};
-
-template <typename T, int DIM>
-__device__ __forceinline__ void restrict_body(const Geom& gf, const Geom& gc, const T* __restrict__ rf,
-                                              T* __restrict__ rc, const ChebStart<T>& cs, int blk) {
-  const long long node = blk * (long long)blockDim.x + threadIdx.x;
-  if (node >= gc.Nv) return;
-  int I, J, K;
-  unflat(node, gc.nv, DIM, I, J, K);
-  const bool con = vnode_constrained(gc, node, I, J, K);
-  T acc[DIM];
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) acc[a] = T(0);
-  if (!con) {
-    int fx[5], fy[5], fz[5];
-    float wx[5], wy[5], wz[5];
-    bool okx[5], oky[5], okz[5];
-    restrict_stencil(I, gf.nv[0], fx, wx, okx);
-    restrict_stencil(J, gf.nv[1], fy, wy, oky);
-    if (DIM == 3) {
-      restrict_stencil(K, gf.nv[2], fz, wz, okz);
-    } else {
-      fz[0] = 0; wz[0] = 1.0f; okz[0] = true;
-    }
-    // the existing fine nodes in slot order (z, then y, then x innermost)
-#pragma unroll
-    for (int k = 0; k < (DIM == 3 ? 5 : 1); ++k) {
-      if (!okz[k]) continue;
-#pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        if (!oky[j]) continue;
-        const T wjk = T(wy[j] * wz[k]);  // exact in float
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-          if (!okx[i]) continue;
-          const long long fn = fx[i] + (long long)gf.nv[0] * (fy[j] + (long long)gf.nv[1] * fz[k]);
-          if (vnode_constrained(gf, fn, fx[i], fy[j], fz[k])) continue;
-          const T w = T(wx[i]) * wjk;
-#pragma unroll
-          for (int a = 0; a < DIM; ++a) acc[a] += w * rf[a * gf.Nv + fn];
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) rc[a * gc.Nv + node] = acc[a];
-  if (cs.d) {
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      const long long i = a * gc.Nv + node;
-      const T v = cs.dinv[i] * acc[a] * cs.inv_theta;
-      cs.d[i] = v;
-      cs.x[i] = v;
-    }
-  }
-}
-
-__device__ __forceinline__ int prolong_stencil(int I, int* ci, float* w) {
-  if (!(I & 1)) { ci[0] = I >> 1; w[0] = 1.0f; return 1; }
-  const int c = I >> 2;  // coarse cell
-  if ((I & 3) == 1) {
-    ci[0] = 2 * c; ci[1] = 2 * c + 1; ci[2] = 2 * c + 2;
-    w[0] = 0.375f; w[1] = 0.75f; w[2] = -0.125f;
-  } else {
-    ci[0] = 2 * c; ci[1] = 2 * c + 1; ci[2] = 2 * c + 2;
-    w[0] = -0.125f; w[1] = 0.75f; w[2] = 0.375f;
-  }
-  return 3;
-}
-
-template <typename T, int DIM>
-__device__ __forceinline__ void prolong_add_body(const Geom& gf, const Geom& gc, const T* __restrict__ xc,
-                                                 T* __restrict__ xf, int blk) {
-  const long long node = blk * (long long)blockDim.x + threadIdx.x;
-  if (node >= gf.Nv) return;
-  int I, J, K;
-  unflat(node, gf.nv, DIM, I, J, K);
-  if (vnode_constrained(gf, node, I, J, K)) return;
-  int cx[3], cy[3], cz[3];
-  float wx[3], wy[3], wz[3];
-  const int mx = prolong_stencil(I, cx, wx);
-  const int my = prolong_stencil(J, cy, wy);
-  int mz = 1;
-  cz[0] = 0; wz[0] = 1.0f;
-  if (DIM == 3) mz = prolong_stencil(K, cz, wz);
-  T acc[DIM];
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) acc[a] = T(0);
-  for (int k = 0; k < mz; ++k)
-    for (int j = 0; j < my; ++j) {
-      const T wjk = T(wy[j] * wz[k]);  // exact in float
-      for (int i = 0; i < mx; ++i) {
-        const long long cn = cx[i] + (long long)gc.nv[0] * (cy[j] + (long long)gc.nv[1] * cz[k]);
-        if (vnode_constrained(gc, cn, cx[i], cy[j], cz[k])) continue;
-        const T w = T(wx[i]) * wjk;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) acc[a] += w * xc[a * gc.Nv + cn];
-      }
-    }
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) xf[a * gf.Nv + node] += acc[a];
-}
-
-template <typename T, int DIM>
-struct RestrictK {
-  using Args = XferArgs<T>;
-  static constexpr int THREADS = TPB, MINB = 1;
-  static __device__ __forceinline__ void body(const Args& a, int blk, int) {
-    restrict_body<T, DIM>(a.gf, a.gc, a.in, a.out, a.cs, blk);
-  }
-};
-template <typename T, int DIM>
-struct ProlongAddK {
-  using Args = XferArgs<T>;
-  static constexpr int THREADS = TPB, MINB = 1;
-  static __device__ __forceinline__ void body(const Args& a, int blk, int) {
-    prolong_add_body<T, DIM>(a.gf, a.gc, a.in, a.out, blk);
-  }
-};
-
-template <typename T>
-cudaError_t launch_restrict(const Geom& gf, const Geom& gc, const T* rf, T* rc, cudaStream_t st, const T* dinv,
-                            T inv_theta, T* d, T* x) {
-  const XferArgs<T> a{gf, gc, rf, rc, ChebStart<T>{dinv, inv_theta, d, x}};
-  if (gf.dim == 2) return submit<RestrictK<T, 2>>(a, nblk(gc.Nv), 0, st);
-  return submit<RestrictK<T, 3>>(a, nblk(gc.Nv), 0, st);
-}
-
-template <typename T>
-cudaError_t launch_prolong_add(const Geom& gf, const Geom& gc, const T* xc, T* xf, cudaStream_t st) {
-  const XferArgs<T> a{gf, gc, xc, xf};
-  if (gf.dim == 2) return submit<ProlongAddK<T, 2>>(a, nblk(gf.Nv), 0, st);
-  return submit<ProlongAddK<T, 3>>(a, nblk(gf.Nv), 0, st);
-}
 
 // ---- pressure mass M_p(1/eta): cell matrix (prod h / 6^d) eta_K^{-1} Pi x Pi (x Pi) ---------------
 template <typename T, int DIM, int MODE>
@@ -371,8 +206,6 @@ cudaError_t launch_pdiag(const Geom& g, const OpCoef<T>& c, const T* eta, T* din
 
 #define INST(T)                                                                                    \
   template cudaError_t launch_diagA<T>(const Geom&, const OpCoef<T>&, const T*, const T*, T*, int, cudaStream_t); \
-  template cudaError_t launch_restrict<T>(const Geom&, const Geom&, const T*, T*, cudaStream_t, const T*, T, T*, T*); \
-  template cudaError_t launch_prolong_add<T>(const Geom&, const Geom&, const T*, T*, cudaStream_t); \
   template cudaError_t launch_pmass<T>(int, PMassArgs<T>, cudaStream_t);                           \
   template cudaError_t launch_pdiag<T>(const Geom&, const OpCoef<T>&, const T*, T*, cudaStream_t);
 INST(float)
