@@ -41,7 +41,7 @@ struct OpCoef {
 template <typename T>
 struct Modal2 {
   T dm[6];               // alpha hx hy M_i M_j w_i w_j by modal2_class(i, j)
-  T dk[2][9];            // component a: hx hy sum_b (1 + [a = b]) K_b / h_b^2 M_other, times the w's
+  T dk[9][2];            // component a: hx hy sum_b (1 + [a = b]) K_b / h_b^2 M_other, times the w's
   T g2[2], g3[2], g23[2];  // divergence: h_other / 24, h_other / 36, h_other / 18
 };
 

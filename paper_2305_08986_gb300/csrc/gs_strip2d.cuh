@@ -332,8 +332,12 @@ __device__ __forceinline__ void strip2d_body(const TileArgs<T>& A, int bid) {
         for (int i = 0; i < 9; ++i)
           if ((cm >> i) & 1u) xl[0][i] = xl[1][i] = T(0);
       }
-      T pl[4], pb[4];
-      cell_modal2<true, false, false>(xl, pl, y, pb, eta, cur.alpha, A.m2);
+      if constexpr (sizeof(T) == 4) {
+        cell_modal2_pair(xl, y, eta, cur.alpha, A.m2);
+      } else {
+        T pl[4], pb[4];
+        cell_modal2<true, false, false>(xl, pl, y, pb, eta, cur.alpha, A.m2);
+      }
     }
     // top node row, unreduced, to the warp above (warp NW - 1: to warp 0 of the next batch, which
     // reads it after the next barrier (A)); slots alternate with the batch parity, and a warp can
@@ -440,8 +444,8 @@ template <typename T, int MODE>
 struct Strip2dK {
   using Args = TileArgs<T>;
   // FP32 A x needs 64 registers with the cells in Legendre modes and runs 4 CTAs per SM: 10.2 -> 7.8 us on
-  // 1280 x 210 cells (11.5 us before); the residual and the Chebyshev step, with their operand windows,
-  // stay at 3 (a smoother call of four steps on 1280 x 224: 85.2 us, 86.5 us at 4, 90.7 us before)
+  // 1280 x 210 cells (11.5 us in 3 x 3 sweeps); the residual and the Chebyshev step, with their operand
+  // windows, stay at 3 (four steps on 1280 x 224: 1.5 % slower at 4)
   static constexpr int THREADS = NT, MINB = sizeof(T) == 4 ? (MODE == TILE_APPLY ? 4 : 3) : 1;
   static __device__ __forceinline__ void body(const Args& a, int blk, int) { strip2d_body<T, MODE>(a, blk); }
 };
