@@ -213,6 +213,11 @@ def krylov_bytes(n: int, iterations: int, restart: int, form: str = "gram"):
     return dots, axpy, fma_dots, fma_axpy
 
 
+# 2D saddle operator in the cells' Legendre modes, an FMA counted as two: modes of 12 node lines 72, diagonal
+# block 56, coupling 20, B^T 24, B 20, back to nodes 72, node sums 13
+SADDLE_FLOPS_PER_CELL = 277
+
+
 def krylov_rooflines(prof: dict, n: int, iterations: int, restart: int, peak_gbs: float, fp64_tflops: float,
                      form: str = "gram"):
     """Achieved GB/s (fraction of the measured HBM peak) and FP64 TFLOP/s (fraction of the measured
@@ -476,7 +481,7 @@ def run_gpu(args, rank, world):
     saddle = None
     if "saddle_fp64" in prof and prof["saddle_fp64"][0] > 0:
         nl, ms = prof["saddle_fp64"]
-        fl = n_cells * (534 + 2 * 75)
+        fl = n_cells * SADDLE_FLOPS_PER_CELL
         ach = fl / (ms / nl * 1e-3) / 1e12
         saddle = {"bound": "alu", "achieved": ach, "peak": args.fp64_peak_tflops, "unit": "TFLOP/s",
                   "frac": ach / args.fp64_peak_tflops, "launches": nl, "avg_launch_us": 1e3 * ms / nl,
@@ -495,12 +500,12 @@ def run_gpu(args, rank, world):
     dominant = roof
     cheb_max = max(cheb_by_kernel.values()) if cheb_by_kernel else 0.0
     if saddle is not None and (roof is None or prof["saddle_fp64"][1] > cheb_max):
-        fl = n_cells * (534 + 2 * 75)
+        fl = n_cells * SADDLE_FLOPS_PER_CELL
         tr = NCU_TRAFFIC_BYTES.get("saddle_fp64")
         dominant = dict(saddle, kernel="saddle_fp64 (FP64 saddle operator of the FGMRES matvec, 32 x 8 cell tiles)",
                         traffic=tr, traffic_over_algorithmic=tr / (8 * 2 * N + 8 * n_cells) if tr else None,
                         flops_per_launch=fl, cheb_step_ms_by_kernel=cheb_by_kernel,
-                        how="algorithmic flops (684 per cell: the sum-factorised A, B and B^T) / average device "
+                        how="algorithmic flops (277 per cell: A, B and B^T in Legendre modes) / average device "
                             "time per launch in the profiled solve; the FP64 pipe is the binding unit")
 
     krylov_table = None

@@ -387,7 +387,7 @@ __device__ __forceinline__ void tile2d_body(const TileArgs<T>& A, int bid) {
 template <typename T, class S2, int MODE, bool WA, bool WBT, bool WB, int CONV = 0>
 struct Tile2dK {
   using Args = TileArgs<T>;
-  // FP64 with B^T (the saddle operator, FP64-pipe-bound): 3 CTAs per SM (76 registers).  1280 x 224: 138 us
+  // FP64 with B^T (the saddle operator, FP64-pipe-bound): 3 CTAs per SM.  1280 x 224: 134 us
   // with the cells in Legendre modes (~180 FP64 operations per cell), 260 us in 3 x 3 sweeps (~400); the
   // FP32 variants stay at 2
   static constexpr int THREADS = S2::NT, MINB = CONV ? 1 : (S2::E0 == 8 ? 8 : (sizeof(T) == 8 && WBT ? 3 : 2));
