@@ -1546,40 +1546,20 @@ gs_status pcheb(gs_ctx* c, int l, const T* b, bool zero_init, bool started = fal
   return GS_OK;
 }
 
-// V-cycle for the pressure Laplacian: input lv.pb, output lv.pxA.  General smoother; pvcycle_deg2 below
-// runs the default one in two launches per level.
+// Whether level l >= 1 of the pressure cycle runs as the two launches of gs_q1cycle.cu: the smoother they are written
+// for, on the levels where they are the faster form (q1cycle_max_nodes in gs_kernels.h).
 template <typename T>
-gs_status pvcycle(gs_ctx* c, int l, bool started = false) {
-  const LevelTag tag__(c, l);
-  Level& lv = c->lv[l];
-  if (l == 0) {
-    if (c->opt.coarse_mode == 1) return pcheb<T>(c, 0, (const T*)lv.pb, true, started);
-    KL(K_SCHUR, launch_coarse_solve<T>(c->PAinv, c->pcfree, c->nfp, (const T*)lv.pb, (T*)lv.pxA, lv.Np, c->pctmp, c->st));
-    return GS_OK;
-  }
-  for (int s = 0; s < c->opt.smooth_steps; ++s) CKS(pcheb<T>(c, l, (const T*)lv.pb, s == 0, s == 0 && started));
-  {
-    PLapArgs<T> a = plap_args<T>(lv);
-    a.x = (const T*)lv.pxA; a.b = (const T*)lv.pb; a.y = (T*)lv.pd;
-    KL(K_SCHUR, launch_plap<T>(TILE_RESID, a, c->st));
-  }
-  Level& cl = c->lv[l - 1];
-  const bool start = c->opt.smooth_steps >= 1 && (l - 1 >= 1 || c->opt.coarse_mode == 1);
-  if (start)
-    KL(K_SCHUR, launch_p_restrict<T>(lv.g, cl.g, lv.pcmask, cl.pcmask, (const T*)lv.pd, (T*)cl.pb, c->st,
-                                     (const T*)cl.pdinv, (T)cheb_inv_theta(cl.plam_hi), (T*)cl.pd, (T*)cl.pxA));
-  else
-    KL(K_SCHUR, launch_p_restrict<T>(lv.g, cl.g, lv.pcmask, cl.pcmask, (const T*)lv.pd, (T*)cl.pb, c->st));
-  CKS(pvcycle<T>(c, l - 1, start));
-  KL(K_SCHUR, launch_p_prolong_add<T>(lv.g, cl.g, lv.pcmask, cl.pcmask, (const T*)cl.pxA, (T*)lv.pxA, c->st));
-  for (int s = 0; s < c->opt.smooth_steps; ++s) CKS(pcheb<T>(c, l, (const T*)lv.pb, false));
-  return GS_OK;
+bool q1cycle_level(const gs_ctx* c, int l) {
+  return l >= 1 && c->opt.smooth_steps == 1 && c->opt.plap_degree == 2 &&
+         c->lv[l].Np <= q1cycle_max_nodes(c->dim, (int)sizeof(T));
 }
 
-// The same cycle for one smoothing step of degree 2 on level l >= 1, right-hand side b
+template <typename T>
+gs_status pvcycle(gs_ctx* c, int l, bool started, const T* b);
+
+// Level l >= 1 of the V-cycle in two launches around the coarser levels
 template <typename T>
 gs_status pvcycle_deg2(gs_ctx* c, int l, const T* b) {
-  const LevelTag tag__(c, l);
   Level& lv = c->lv[l];
   Level& cl = c->lv[l - 1];
   const PLapArgs<T> p = plap_args<T>(lv);
@@ -1596,13 +1576,41 @@ gs_status pvcycle_deg2(gs_ctx* c, int l, const T* b) {
     a.sd = (T*)cl.pd; a.sx = (T*)cl.pxA; a.sdinv = (const T*)cl.pdinv; a.s_inv_theta = (T)cheb_inv_theta(cl.plam_hi);
   }
   KL(K_SCHUR, launch_q1cycle<T>(0, a, c->st));
-  if (l > 1)
-    CKS(pvcycle_deg2<T>(c, l - 1, (const T*)cl.pb));
-  else
-    CKS(pvcycle<T>(c, 0, start));
+  CKS(pvcycle<T>(c, l - 1, start, (const T*)cl.pb));
   a.e = (const T*)cl.pxA; a.xout = (T*)lv.pxB;
   KL(K_SCHUR, launch_q1cycle<T>(1, a, c->st));
   std::swap(lv.pxA, lv.pxB);
+  return GS_OK;
+}
+
+// V-cycle for the pressure Laplacian: right-hand side b (zero on constrained entries, except where the level runs in
+// two launches, which take them as zero), output lv.pxA.  started: the smoother's first step from zero is done.
+template <typename T>
+gs_status pvcycle(gs_ctx* c, int l, bool started, const T* b) {
+  const LevelTag tag__(c, l);
+  Level& lv = c->lv[l];
+  if (l == 0) {
+    if (c->opt.coarse_mode == 1) return pcheb<T>(c, 0, b, true, started);
+    KL(K_SCHUR, launch_coarse_solve<T>(c->PAinv, c->pcfree, c->nfp, b, (T*)lv.pxA, lv.Np, c->pctmp, c->st));
+    return GS_OK;
+  }
+  if (q1cycle_level<T>(c, l)) return pvcycle_deg2<T>(c, l, b);
+  for (int s = 0; s < c->opt.smooth_steps; ++s) CKS(pcheb<T>(c, l, b, s == 0, s == 0 && started));
+  {
+    PLapArgs<T> a = plap_args<T>(lv);
+    a.x = (const T*)lv.pxA; a.b = b; a.y = (T*)lv.pd;
+    KL(K_SCHUR, launch_plap<T>(TILE_RESID, a, c->st));
+  }
+  Level& cl = c->lv[l - 1];
+  const bool start = c->opt.smooth_steps >= 1 && (l == 1 ? c->opt.coarse_mode == 1 : !q1cycle_level<T>(c, l - 1));
+  if (start)
+    KL(K_SCHUR, launch_p_restrict<T>(lv.g, cl.g, lv.pcmask, cl.pcmask, (const T*)lv.pd, (T*)cl.pb, c->st,
+                                     (const T*)cl.pdinv, (T)cheb_inv_theta(cl.plam_hi), (T*)cl.pd, (T*)cl.pxA));
+  else
+    KL(K_SCHUR, launch_p_restrict<T>(lv.g, cl.g, lv.pcmask, cl.pcmask, (const T*)lv.pd, (T*)cl.pb, c->st));
+  CKS(pvcycle<T>(c, l - 1, start, (const T*)cl.pb));
+  KL(K_SCHUR, launch_p_prolong_add<T>(lv.g, cl.g, lv.pcmask, cl.pcmask, (const T*)cl.pxA, (T*)lv.pxA, c->st));
+  for (int s = 0; s < c->opt.smooth_steps; ++s) CKS(pcheb<T>(c, l, b, false));
   return GS_OK;
 }
 
@@ -1611,10 +1619,9 @@ gs_status pvcycle_deg2(gs_ctx* c, int l, const T* b) {
 template <typename T>
 gs_status plap_inverse(gs_ctx* c, const T* r) {
   Level& F = c->lv[c->L - 1];
-  if (c->L > 1 && c->opt.smooth_steps == 1 && c->opt.plap_degree == 2) return pvcycle_deg2<T>(c, c->L - 1, r);
+  if (q1cycle_level<T>(c, c->L - 1)) return pvcycle<T>(c, c->L - 1, false, r);
   KL(K_VEC, launch_mask_copy<T>(r, F.pcmask, (T*)F.pb, F.Np, c->st));
-  CKS(pvcycle<T>(c, c->L - 1));
-  return GS_OK;
+  return pvcycle<T>(c, c->L - 1, false, (const T*)F.pb);
 }
 
 // ---- saddle-point multigrid with the block smoother K_j (Sec. 4, Eq. "smoother") ---------------

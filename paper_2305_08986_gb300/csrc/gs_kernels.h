@@ -192,6 +192,11 @@ struct Q1CycleArgs {
 };
 template <typename T>
 cudaError_t launch_q1cycle(int up, const Q1CycleArgs<T>& a, cudaStream_t st);
+// largest level (pressure nodes) that the cycle runs in these two launches; larger ones take one launch per step
+// (gs_q1cycle.cu has the figures)
+constexpr long long q1cycle_max_nodes(int dim, int bytes) {
+  return dim == 2 ? (bytes == 4 ? (1LL << 62) : (1LL << 17)) : (bytes == 4 ? (1LL << 18) : 0);
+}
 // out[i] = mask[i] ? 0 : in[i]   (may run in place)
 template <typename T>
 cudaError_t launch_mask_copy(const T* in, const uint8_t* mask, T* out, long long n, cudaStream_t st);

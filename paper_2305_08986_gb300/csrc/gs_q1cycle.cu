@@ -4,11 +4,18 @@
 //   up    x <- x + P e;  d = D^-1 (b - K x) / theta, x <- x + d;  x <- x + c1 d + c2 D^-1 (b - K x)
 // (K: the operator of gs_q1tile.cu, R / P: bilinear transfers; entries with a mask are zero throughout.)
 //
-// The levels of this cycle hold 0.3 to 290,000 nodes, and a launch costs 2.5 to 3 us whatever it holds, so the
+// The levels of this cycle hold 328 to 290,000 nodes, and a launch costs 2.5 to 3 us whatever it holds, so the
 // cycle was bound by its launches, seven per level.  A CTA evaluates a box of nodes with the halo that the
 // following stages need (3 nodes down, 2 up) in shared memory and repeats the halo's work of its neighbours:
 // 1.9 (2D) or 6 (3D) node evaluations per node instead of one, against five launches and as many passes over memory.
 // Pressure V-cycle on the 1280 x 224 hierarchy (FP32, six levels): 99.9 -> 54.9 us; channel solve 38.8 -> 37.0 ms.
+//
+// The repeated evaluations are worth it while launches bound the level (q1cycle_max_nodes in gs_kernels.h).  One cycle
+// with the finest level in two launches / in seven, us:
+//   2D FP32  512^2 66 / 78, 2048^2 312 / 375: every level in two
+//   2D FP64  320^2 136 / 138, 384^2 169 / 166, 512^2 223 / 212, 768^2 366 / 333: up to 2^17 nodes
+//   3D FP32  48^3 75 / 82, 56^3 78 / 82, 64^3 105 / 103, 80^3 148 / 135: up to 2^18 nodes
+//   3D FP64  8^3 66 / 49, 32^3 244 / 208 (all levels in seven: 172): the FP64 pipe bounds even the smallest; none
 #include "gs_kernels.h"
 
 namespace gs {
