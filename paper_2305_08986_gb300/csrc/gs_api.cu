@@ -70,6 +70,10 @@ struct Level {
   Geom g{};
   OpCoef<double> c64{};
   OpCoef<float> c32{};
+  Modal2<double> m2_64{};  // the cell operators' coefficients in Legendre modes, 2D and 3D
+  Modal2<float> m2_32{};
+  ModalCoef<double> m3_64{};
+  ModalCoef<float> m3_32{};
   double* eta64 = nullptr;
   float* eta32 = nullptr;
   double* alpha64 = nullptr;  // alpha per cell, or NULL (alpha then lives in the coefficients)
@@ -769,8 +773,16 @@ void set_geom(gs_ctx* c, const gs_mesh* m) {
     g.cvoid = lv.cvoid;
     g.ccmask = lv.ccmask;
     // alpha per cell: the coefficients carry alpha = 1 and the kernels multiply by alpha_K
-    lv.c64 = make_coef<double>(c->dim, lv.h, c->alpha_cells ? 1.0 : c->alpha);
-    lv.c32 = make_coef<float>(c->dim, lv.h, c->alpha_cells ? 1.0 : c->alpha);
+    const double alpha = c->alpha_cells ? 1.0 : c->alpha;
+    lv.c64 = make_coef<double>(c->dim, lv.h, alpha);
+    lv.c32 = make_coef<float>(c->dim, lv.h, alpha);
+    if (c->dim == 2) {
+      lv.m2_64 = make_modal2<double>(lv.h, alpha);
+      lv.m2_32 = make_modal2<float>(lv.h, alpha);
+    } else {
+      lv.m3_64 = make_modal<double>(lv.h, alpha);
+      lv.m3_32 = make_modal<float>(lv.h, alpha);
+    }
     // Q1 stiffness coefficients kc[a] = prod_{b != a} h_b / (6^(d-1) h_a)
     for (int a = 0; a < 3; ++a) {
       if (a >= c->dim) { lv.pkc[a] = 0.0; continue; }
@@ -789,6 +801,8 @@ template <>
 OpCoef<double> coef<double>(const Level& lv) { return lv.c64; }
 template <>
 OpCoef<float> coef<float>(const Level& lv) { return lv.c32; }
+inline void set_modal(TileArgs<double>& a, const Level& lv) { a.m2 = lv.m2_64; a.m3 = &lv.m3_64; }
+inline void set_modal(TileArgs<float>& a, const Level& lv) { a.m2 = lv.m2_32; a.m3 = &lv.m3_32; }
 template <typename T>
 const T* etap(const Level& lv);
 template <>
@@ -808,6 +822,7 @@ TileArgs<T> tile_args(const Level& lv) {
   TileArgs<T> a{};
   a.g = lv.g;
   a.c = coef<T>(lv);
+  set_modal(a, lv);
   a.eta = etap<T>(lv);
   a.alpha = alphap<T>(lv);
   a.shape = lv.shape;
@@ -2919,6 +2934,11 @@ gs_status gs_lift_rhs(gs_ctx* c, const double* f, const double* g, double* rhs) 
     TileArgs<double> a = tile_args<double>(F);
     a.c = make_coef<double>(c->dim, F.h, 1.0);
     a.c.eta_scale = 0.0;
+    ModalCoef<double> m3;
+    if (c->dim == 2)
+      a.m2 = make_modal2<double>(F.h, 1.0);
+    else
+      m3 = make_modal<double>(F.h, 1.0), a.m3 = &m3;
     a.conv = 0;  // the load is the plain mass (the corrector terms belong to the operator)
     a.xu = f; a.yu = c->t1; a.raw = 1;
     CK(launch_tile<double>(c->dim, TILE_APPLY, OPS_A, a, c->st));

@@ -37,14 +37,6 @@ struct OpCoef {
   T pm;
 };
 
-// Coefficients of the 2D cell operators in the cells' Legendre modes (gs_modal.cuh), mode i + 3 j.
-template <typename T>
-struct Modal2 {
-  T dm[6];               // alpha hx hy M_i M_j w_i w_j by modal2_class(i, j)
-  T dk[9][2];            // component a: hx hy sum_b (1 + [a = b]) K_b / h_b^2 M_other, times the w's
-  T g2[2], g3[2], g23[2];  // divergence: h_other / 24, h_other / 36, h_other / 18
-};
-
 __host__ __device__ inline bool face_constrained(const Geom& g, int I, int J, int K) {
   unsigned f = g.faces;
   if ((f & 1u) && I == 0) return true;

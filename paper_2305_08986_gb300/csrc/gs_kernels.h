@@ -4,6 +4,7 @@
 
 #include "gs_batch.cuh"
 #include "gs_common.cuh"
+#include "gs_modal_coef.h"
 
 namespace gs {
 
@@ -19,7 +20,8 @@ template <typename T>
 struct TileArgs {
   Geom g;
   OpCoef<T> c;
-  Modal2<T> m2;   // 2D: coefficients in the cells' modes (set by the launcher)
+  Modal2<T> m2;   // 2D: coefficients in the cells' modes
+  const ModalCoef<T>* m3;  // 3D: the same (host memory, read by the launcher)
   const T* eta;   // per cell
   const T* alpha; // per cell factor of the mass term (alpha_K; NULL: 1, alpha then lives in c.mm)
   const T* xu;    // velocity input (A and B), CHEB: current iterate

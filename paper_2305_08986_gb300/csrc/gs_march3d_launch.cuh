@@ -62,7 +62,7 @@ cudaError_t launch(const TileArgs<T>& a, cudaStream_t st) {
   if (s.px < 1) return cudaErrorInvalidValue;
   March3Args<T> m;
   m.t = a;
-  m.m = make_modal<T>(a.g, a.c);
+  m.m = *a.m3;
   m.px = s.px;
   m.py = s.py;
   m.np0 = s.np0;

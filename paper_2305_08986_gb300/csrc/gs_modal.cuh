@@ -20,63 +20,6 @@
 
 namespace gs {
 
-// Coefficients of one level (see make_modal).  Mode index q = i + 3 j (+ 9 k), x fastest.
-template <typename T>
-struct ModalCoef {
-  T dm[10];      // alpha prod h prod_a M_a w_a, by the numbers of 1s and 2s among the mode's indices
-  T dk[3][27];   // component a: prod h sum_b (1 + [a = b]) K_b / h_b^2 prod_{c != b} M_c, times the w's
-  T dc[3][3];    // coupling of the two components other than p: h_p M_k w_k / 36 (2D: dc[2][0] = 1/36)
-  T g2[3], g3[3], g23[3];  // divergence: g_a / 2, g_a / 3, 2 g_a / 3 with g_a = prod_{b != a} h_b / 12
-};
-
-// position of a mode in dm: (number of indices equal to 1, number equal to 2)
-__host__ __device__ constexpr int modal_class(int i, int j, int k) {
-  const int n1 = (i == 1) + (j == 1) + (k == 1), n2 = (i == 2) + (j == 2) + (k == 2);
-  return n2 == 0 ? n1 : (n2 == 1 ? 4 + n1 : (n2 == 2 ? 7 + n1 : 9));
-}
-
-template <typename T>
-inline ModalCoef<T> make_modal(const Geom& g, const OpCoef<T>& c) {
-  const int dim = g.dim;
-  const double M[3] = {1.0 / 36.0, 1.0 / 12.0, 1.0 / 45.0}, K[3] = {0.0, 1.0, 4.0 / 3.0}, w[3] = {1.0, 1.0, 2.0};
-  ModalCoef<T> m{};
-  double vol = 1.0;
-  for (int a = 0; a < dim; ++a) vol *= g.h[a];
-  const double av = (double)c.mm * (dim == 2 ? 900.0 : 27000.0);  // alpha prod h
-  for (int k = 0; k < (dim == 3 ? 3 : 1); ++k)
-    for (int j = 0; j < 3; ++j)
-      for (int i = 0; i < 3; ++i) {
-        const int ix[3] = {i, j, k};
-        double ww = 1.0, mm = 1.0;
-        for (int a = 0; a < dim; ++a) {
-          ww *= w[ix[a]];
-          mm *= M[ix[a]];
-        }
-        m.dm[modal_class(i, j, dim == 3 ? k : 0)] = (T)(av * mm * ww);
-        for (int comp = 0; comp < dim; ++comp) {
-          double s = 0.0;
-          for (int b = 0; b < dim; ++b) {
-            double t = (b == comp ? 2.0 : 1.0) * K[ix[b]] / (g.h[b] * g.h[b]);
-            for (int e = 0; e < dim; ++e)
-              if (e != b) t *= M[ix[e]];
-            s += t;
-          }
-          m.dk[comp][i + 3 * j + 9 * k] = (T)(vol * s * ww);
-        }
-      }
-  for (int p = 0; p < 3; ++p)
-    for (int k = 0; k < 3; ++k) m.dc[p][k] = (T)(dim == 3 ? g.h[p] * M[k] * w[k] / 36.0 : (k == 0 ? 1.0 / 36.0 : 0.0));
-  for (int a = 0; a < dim; ++a) {
-    double ga = 1.0;
-    for (int b = 0; b < dim; ++b)
-      if (b != a) ga *= g.h[b] / 12.0;
-    m.g2[a] = (T)(ga / 2.0);
-    m.g3[a] = (T)(ga / 3.0);
-    m.g23[a] = (T)(2.0 * ga / 3.0);
-  }
-  return m;
-}
-
 template <typename T>
 __device__ __forceinline__ void to_modes(T x0, T x1, T x2, T& a0, T& a1, T& a2) {
   const T s = x0 + x2;
@@ -112,27 +55,13 @@ __device__ __forceinline__ void plane_from_modes(T (&v)[9]) {
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
-// position of a 2D mode (i, j) in Modal2::dm (symmetric in i and j)
-__host__ __device__ constexpr int modal2_class(int i, int j) {
-  const int lo = i < j ? i : j, hi = i < j ? j : i;
-  return lo == 0 ? hi : (lo == 1 ? 2 + hi : 5);
+// (alpha mass + eta viscous) coefficient of mode q >= 1, component c; ms: the mass part.  FP32: with the remainder of
+// the viscous coefficient (gs_modal_coef.h).
+__device__ __forceinline__ float modal2_diag(const Modal2<float>& m, int q, int c, float eta, float ms) {
+  return fmaf(eta, m.dk[q][c], fmaf(eta, m.dl[q][c], ms));
 }
-
-template <typename T>
-inline Modal2<T> make_modal2(const Geom& g, const OpCoef<T>& c) {
-  const ModalCoef<T> m = make_modal<T>(g, c);
-  Modal2<T> q{};
-  for (int j = 0; j < 3; ++j)
-    for (int i = 0; i < 3; ++i) {
-      q.dm[modal2_class(i, j)] = m.dm[modal_class(i, j, 0)];
-      for (int a = 0; a < 2; ++a) q.dk[i + 3 * j][a] = m.dk[a][i + 3 * j];
-    }
-  for (int a = 0; a < 2; ++a) {
-    q.g2[a] = m.g2[a];
-    q.g3[a] = m.g3[a];
-    q.g23[a] = m.g23[a];
-  }
-  return q;
+__device__ __forceinline__ double modal2_diag(const Modal2<double>& m, int q, int c, double eta, double ms) {
+  return fma(eta, m.dk[q][c], ms);
 }
 
 // r += coupling of the two components in the modes of one 2D cell: mode (0|1, 1|2) of component x with (+1, -1) of
@@ -206,7 +135,8 @@ __device__ __forceinline__ void cell_modal2_pair(const float (&x)[2][9], float (
     const float ms = mul_rn(alpha, m.dm[modal2_class(q % 3, q / 3)]);
     const f32x2 mm = pack2(ms, ms);
     unpack2(v[q], a[0][q], a[1][q]);
-    unpack2(mul2(q == 0 ? mm : fma2(e, pack2(m.dk[q][0], m.dk[q][1]), mm), v[q]), r[0][q], r[1][q]);
+    const f32x2 d = q == 0 ? mm : fma2(e, pack2(m.dk[q][0], m.dk[q][1]), fma2(e, pack2(m.dl[q][0], m.dl[q][1]), mm));
+    unpack2(mul2(d, v[q]), r[0][q], r[1][q]);
   }
   modal2_couple(a, r, eta);
 #pragma unroll
@@ -239,7 +169,7 @@ __device__ __forceinline__ void cell_modal2(const T (&x)[2][9], const T (&p)[4],
 #pragma unroll
       for (int q = 0; q < 9; ++q) {
         const T ms = mul_rn(alpha, m.dm[modal2_class(q % 3, q / 3)]);
-        r[c][q] = mul_rn(q == 0 ? ms : fma(eta, m.dk[q][c], ms), a[c][q]);
+        r[c][q] = mul_rn(q == 0 ? ms : modal2_diag(m, q, c, eta, ms), a[c][q]);
       }
     modal2_couple(a, r, eta);
   } else if (WBT) {

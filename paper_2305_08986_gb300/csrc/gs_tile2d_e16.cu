@@ -21,7 +21,6 @@ namespace gs {
 template <typename T>
 cudaError_t launch_tile2d(int mode, int ops, TileArgs<T> a, cudaStream_t st) {
   if (mode == TILE_CHEB && ops != OPS_A) return cudaErrorInvalidValue;
-  a.m2 = make_modal2<T>(a.g, a.c);
   // corrector stage: launches that include the velocity block take the convection terms (32 x 8
   // tiles); B and B^T alone are unchanged
   if (a.conv && (ops & OPS_A)) return launch_tile2d_conv<T>(mode, ops, a, st);
