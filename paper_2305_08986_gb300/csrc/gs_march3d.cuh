@@ -33,6 +33,7 @@ struct March3Args {
   int px, py;      // threads (cells) of a patch along x and y
   int np0, np1;    // patches along x and y
   int layers;      // evaluated cell layers per segment
+  int skip;        // warps without a column only keep the barriers
 };
 
 namespace march3 {
@@ -40,6 +41,7 @@ template <typename T>
 struct Cfg {
   static constexpr int NT = 128;   // threads per CTA
   static constexpr int MINB = 2;   // CTAs per SM: 8 warps at 255 registers; 12 at 168 spilled (4 Chebyshev steps, 64^3: 23 % slower)
+  static constexpr double SHARE = sizeof(T) == 4 ? 0.5 : 0.9;  // of an SM's issue (FP64: pipe) slots a CTA takes
 };
 
 // values per thread: exchanged with the neighbours per layer; epilogue operands of the 8 nodes a cell owns
@@ -87,6 +89,14 @@ __device__ __forceinline__ void body(const March3Args<T>& M, int bid) {
   const bool own = here && (left || p0 == 0) && (below || p1 == 0);
   const bool two0 = c0 < n0, two1 = c1 < n1;      // node columns / rows owned besides the first
   const int zs = sg * (M.layers - 1), ze = min(n2, zs + M.layers);
+  const int zend = ze == n2 ? n2 + 1 : ze;  // one extra pass after the mesh's last layer completes the top node plane
+  // In a launch with other meshes' blocks a warp without a column (a patch may hold fewer than 128) only keeps the
+  // barriers: its arithmetic would take their issue slots (64 systems of 16^3: 127 -> 117 ms).  Alone it runs along, and
+  // its instruction fetches serve the others: 4 Chebyshev steps on 8^3, FP32, take 32 us, and 39 us without it.
+  if (M.skip && !__any_sync(0xffffffffu, here)) {
+    for (int c2 = zs; c2 < zend; ++c2) __syncthreads();
+    return;
+  }
   // byte offsets in a plane (planes are below 4 GB): the cell's three node rows (threads without a cell read some
   // cell of the mesh), and the two node rows a thread writes
   const long long vcol = 2 * min(c0, n0) + (long long)nv0 * (2 * min(c1, n1));
@@ -180,8 +190,6 @@ __device__ __forceinline__ void body(const March3Args<T>& M, int bid) {
   T xm[3][9], xt[3][9];  // the layer's middle and top node planes
   unsigned pmm = plane_mask(2 * zs + 1), pmt = plane_mask(2 * zs + 2);
 
-  // one extra pass after the mesh's last layer completes the top node plane
-  const int zend = ze == n2 ? n2 + 1 : ze;
 #pragma unroll 1
   for (int c2 = zs; c2 < zend; ++c2) {
     T bot[3][9], mid[3][9], pb[4];
