@@ -12,8 +12,9 @@ cudaError_t launch(const TileArgs<T>& a, cudaStream_t st) {
   using K = March3K<T, MODE, WA, WBT, WB>;
   constexpr size_t smem = sizeof(T) * (2 * exchange_values<WA || WBT, WB>() + operand_values<MODE, WA || WBT>()) * Cfg<T>::NT;
   const bool shared = current_recorder() != nullptr;  // recorded into a launch of several meshes
-  const Shape s = choose(a.g.n, Cfg<T>::NT, Cfg<T>::SHARE, sm_count(), ctas_per_sm<K>(smem), a.shape == 1 ? 4 : a.g.n[2],
-                         shared);
+  thread_local Answers shapes;
+  const Shape& s = shapes.find({{a.g.n[0], a.g.n[1], a.g.n[2]}, Cfg<T>::NT, sm_count(), ctas_per_sm<K>(smem),
+                                a.shape == 1 ? 4 : a.g.n[2], Cfg<T>::SHARE, shared});
   if (s.px < 1) return cudaErrorInvalidValue;
   March3Args<T> m;
   m.t = a;

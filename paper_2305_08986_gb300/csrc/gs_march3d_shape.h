@@ -61,5 +61,35 @@ inline Shape choose(const int* cells, int threads, double share, int sms, int re
   return best;
 }
 
+// The same from the last few answers of the calling thread: the search takes 3 to 5 us of a host core, as long as a
+// small launch, and depends on its arguments alone.  (One list per kernel and thread; 32 entries hold the levels of
+// several contexts.)
+struct Query {
+  int cells[3], threads, sms, resident, max_layers;
+  double share;
+  bool shared;
+  bool operator==(const Query& o) const {
+    return cells[0] == o.cells[0] && cells[1] == o.cells[1] && cells[2] == o.cells[2] && threads == o.threads &&
+           sms == o.sms && resident == o.resident && max_layers == o.max_layers && share == o.share && shared == o.shared;
+  }
+};
+struct Answers {
+  static constexpr int N = 32;
+  Query q[N] = {};
+  Shape s[N] = {};
+  int next = 0;
+  long long searches = 0;
+  const Shape& find(const Query& k) {
+    for (int i = 0; i < N; ++i)
+      if (q[i] == k) return s[i];  // an empty entry has threads = 0 and equals no query
+    const int i = next;
+    next = (next + 1) % N;
+    searches++;
+    q[i] = k;
+    s[i] = choose(k.cells, k.threads, k.share, k.sms, k.resident, k.max_layers, k.shared);
+    return s[i];
+  }
+};
+
 }  // namespace march3
 }  // namespace gs

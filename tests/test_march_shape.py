@@ -10,6 +10,8 @@ import subprocess
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+# meshes with several patches along both axes, whose segments by size have more than four layers (the first in FP64 only)
+SEVERAL_PATCHES = [(28, 64, 40), (33, 50, 60)]
 DRIVER = r"""
 #include <cstdio>
 #include "gs_march3d_shape.h"
@@ -18,8 +20,11 @@ int main() {
   int c[3], res, cap, shared;
   double share;
   while (std::scanf("%d %d %d %d %d %lf %d", c, c + 1, c + 2, &res, &cap, &share, &shared) == 7) {
-    const Shape s = choose(c, 128, share, 152, res, cap, shared != 0);
-    std::printf("%d %d %d %d %d %d %lld\n", s.px, s.py, s.np0, s.np1, s.layers, s.segs, work(s));
+    static Answers a;
+    const Shape s = a.find({{c[0], c[1], c[2]}, 128, 152, res, cap, share, shared != 0});
+    const Shape t = choose(c, 128, share, 152, res, cap, shared != 0);
+    const bool same = s.px == t.px && s.py == t.py && s.layers == t.layers && s.segs == t.segs;
+    std::printf("%d %d %d %d %d %d %lld %lld %d\n", s.px, s.py, s.np0, s.np1, s.layers, s.segs, work(s), a.searches, same);
   }
 }
 """
@@ -57,3 +62,23 @@ def test_small_meshes_execute_little_beyond_their_cells(choose):
     q = [(n, n, n, 2, n, share, 1) for n in (8, 12, 16, 20, 24, 28, 32) for share in (0.5, 0.9)]
     for (n, *_), s in zip(q, choose(q)):
         assert 32 * s[6] <= 3 * n ** 3
+
+
+def test_answers_are_kept_and_keyed_by_every_argument(choose):
+    """One search per distinct query while they fit the list, the searched shape in every answer, also beyond it."""
+    q = [(a, 24, c, res, cap, share, shared) for a in (8, 24) for c in (16, 64) for res, cap in ((2, c), (2, 4), (1, c))
+         for share, shared in ((0.5, 0), (0.5, 1))]
+    rows = choose(q * 5)
+    assert len(set(q)) == len(q) <= 32 and rows[-1][7] == len(q)
+    rows = choose([(n, n, n, 2, n, 0.5, 0) for n in list(range(8, 60)) * 2])
+    assert all(r[8] for r in rows)
+
+
+def test_larger_meshes_get_other_shapes_by_size_than_with_four_layers(choose):
+    """What tests/test_gpu_march_shapes.py relies on."""
+    for n in SEVERAL_PATCHES:
+        for share in (0.5, 0.9):
+            by_size, four = choose([n + (2, n[2], share, 0), n + (2, 4, share, 0)])
+            assert by_size[2] > 1 and by_size[3] > 1 and four[4] <= 4
+            if share == 0.9 or n != SEVERAL_PATCHES[0]:
+                assert by_size[4] > 4
