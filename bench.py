@@ -868,8 +868,7 @@ def run_extension(args):
             e.record(st)
             e.synchronize()
             ts.append(a.elapsed_time(e))
-        key = ("fp32_multigrid" if prec == 32 else "fp64_multigrid") + ("_kA6" if kdeg == 6 else "")
-        out[key] = {
+        out["fp32_multigrid" if prec == 32 else "fp64_multigrid"] = {
             "time_to_solve_ms": statistics.median(ts), "iterations": it, "rel_residual": rr, "unknowns": s.n_u}
         s.close()
     print(json.dumps(out), flush=True)
