@@ -427,13 +427,13 @@ __device__ __forceinline__ void cell_A3p(const T* xc, const T* x1, const T* x2, 
 // B^T contribution to output component "logical x" in the rotated frame: -bd_a (Gi^T along x, Ni^T
 // along y and z) applied to the cell's pressure nodes given in the logical frame
 template <typename T>
-__device__ __forceinline__ void cell_BT3p(const T (&p)[8], T (&u)[27], T bd_a, bool acc) {
+__device__ __forceinline__ void cell_BT3p(const T (&p)[8], T (&u)[27], T bd_a) {
   T a[12], b[18], v[27];
   sweep<OpNT, 2, 2, 2, 2, false>(p, a);  // (2,2,3)
   sweep<OpNT, 1, 2, 2, 3, false>(a, b);  // (2,3,3)
   sweep<OpGT, 0, 2, 3, 3, false>(b, v);  // (3,3,3)
 #pragma unroll
-  for (int i = 0; i < 27; ++i) u[i] = (acc ? u[i] : T(0)) - bd_a * v[i];
+  for (int i = 0; i < 27; ++i) u[i] -= bd_a * v[i];
 }
 
 // (B u) of one 3D cell with the velocity read from a shared-memory window:

@@ -19,13 +19,10 @@
 
 namespace gs {
 
-// Tile shapes: TC0 x TC1 x TC2 evaluated cells ((TC - 1) owned per axis), one thread per
-// (2 x 2 x 2 group, output component).  The skewed shared-memory layouts below assume TC0 = TC1 =
-// 8; TC2 may be 8 or 4 (a warp then covers the same group pattern).
-template <int C2>
+// Tile: 8 x 8 x 4 evaluated cells (7 x 7 x 3 owned), one thread per (2 x 2 x 2 group, output component): 96 threads.
+// Deeper tiles do not fit the shared memory that the window of v° takes as well.
 struct TileShape3 {
-  static_assert(C2 == 8 || C2 == 4, "3D tile depth");
-  static constexpr int TC0 = 8, TC1 = 8, TC2 = C2;
+  static constexpr int TC0 = 8, TC1 = 8, TC2 = 4;
   static constexpr int G0 = TC0 / 2, G1 = TC1 / 2, G2 = TC2 / 2;
   static constexpr int SPLIT = 3;
   static constexpr int NG = G0 * G1 * G2;
@@ -71,10 +68,11 @@ struct Skew3 {
   static constexpr int OA = 1, OB = F ? 0 : 3, OP = F ? 236 : 229;  // output tile (VE = 15)
 };
 
-template <typename T, int MODE, bool WA, bool WBT, bool WB, class S, int CONV = 0>
+// SADDLE: with B^T p in the velocity rows and the pressure rows B u
+template <typename T, bool SADDLE>
 struct Smem3 {
   using K = Skew3<T>;
-  static constexpr bool NEED_U = WA || WB, WU = WA || WBT;
+  using S = TileShape3;
   static constexpr int W0 = 2 * S::TC0 + 1, W1 = 2 * S::TC1 + 1, W2 = 2 * S::TC2 + 1;  // staged velocity window
   static constexpr int W = W0, WV = W0 * W1 * W2;
   static constexpr int WVA = (W0 - 1) + (W1 - 1) * W + (W2 - 1) * K::WP + K::WA * ((W1 - 1) >> 2) +
@@ -83,24 +81,24 @@ struct Smem3 {
                               K::OA * ((S::VE1 - 1) >> 2) + K::OB * ((S::VE2 - 1) >> 2) + 1;
   static constexpr int PW0 = S::TC0 + 1, PW1 = S::TC1 + 1, PW2 = S::TC2 + 1;
   static constexpr int PWV = PW0 * PW1 * PW2;               // staged pressure window
-  static constexpr int SU = WU ? 3 * VSZA : 0;              // velocity outputs
-  static constexpr int SP = WB ? S::PSZ : 0;                // pressure outputs
-  static constexpr int SX = NEED_U ? 3 * WVA : 0;
-  static constexpr int SPW = WBT ? PWV : 0;
-  static constexpr int SV = CONV ? 3 * WVA : 0;              // v° window (corrector stage)
+  static constexpr int SU = 3 * VSZA;                       // velocity outputs
+  static constexpr int SP = SADDLE ? S::PSZ : 0;            // pressure outputs
+  static constexpr int SX = 3 * WVA;
+  static constexpr int SPW = SADDLE ? PWV : 0;
+  static constexpr int SV = 3 * WVA;                         // v° window
   static constexpr int TOTAL = SU + SP + SX + SPW + SV;      // elements of T
-  static constexpr int FLAGS = NEED_U ? WV : 0;              // bytes
+  static constexpr int FLAGS = WV;                           // bytes
   static_assert(S::TC0 == 8 && S::TC1 == 8, "the skewed layouts assume 8 x 8 cells in x and y");
   static_assert(K::WP >= W * W1 + K::WA * ((W1 - 1) >> 2) && K::OP >= S::VE0 * S::VE1 + K::OA * ((S::VE1 - 1) >> 2),
                 "planes of the skewed layouts must not overlap");
 };
 
-template <typename T, int MODE, bool WA, bool WBT, bool WB, class S, int CONV = 0>
+template <typename T, int MODE, bool SADDLE, int CONV>
 __device__ __forceinline__ void tile3d_body(const TileArgs<T>& A, int bid) {
+  using S = TileShape3;
   using D = S;
-  using SM = Smem3<T, MODE, WA, WBT, WB, S, CONV>;
+  using SM = Smem3<T, SADDLE>;
   using K = Skew3<T>;
-  constexpr bool NEED_U = SM::NEED_U, WU = SM::WU;
   constexpr int W = SM::W, WW = W * SM::W1, WV = SM::WV, WVA = SM::WVA, VSZA = SM::VSZA;
   constexpr int PW0 = SM::PW0, PW01 = SM::PW0 * SM::PW1;
   auto widx = [](int i0, int i1, int i2) { return i0 + W * i1 + K::WP * i2 + K::WA * (i1 >> 2) + K::WB * (i2 >> 2); };
@@ -112,7 +110,7 @@ __device__ __forceinline__ void tile3d_body(const TileArgs<T>& A, int bid) {
   T* sp = su + SM::SU;
   T* sx = sp + SM::SP;
   T* spw = sx + SM::SX;
-  T* svc = spw + SM::SPW;  // v° window (CONV)
+  T* svc = spw + SM::SPW;  // v° window
   uint8_t* sflag = reinterpret_cast<uint8_t*>(svc + SM::SV);
   const Geom& g = A.g;
   const OpCoef<T>& c = A.c;
@@ -135,25 +133,22 @@ __device__ __forceinline__ void tile3d_body(const TileArgs<T>& A, int bid) {
   const long long Nv = g.Nv;
 
   // ---- stage the windows (all copies in flight together), zero the output tiles ----
-  if (NEED_U) {
-    const int I0 = 2 * (cs0 - 1), J0 = 2 * (cs1 - 1), K0 = 2 * (cs2 - 1);
-    for (int i = tid; i < WV; i += D::THREADS) {
-      const int a = i % W, b = (i / W) % SM::W1, k = i / WW;
-      const int I = I0 + a, J = J0 + b, K = K0 + k;
-      const bool inr = I >= 0 && I < g.nv[0] && J >= 0 && J < g.nv[1] && K >= 0 && K < g.nv[2];
-      const long long node = inr ? I + (long long)g.nv[0] * (J + (long long)g.nv[1] * K) : 0;
-      const bool fcon = !raw && inr && !vmasked && face_constrained(g, I, J, K);
-      const int wi = widx(a, b, k);
+  const int I0 = 2 * (cs0 - 1), J0 = 2 * (cs1 - 1), K0 = 2 * (cs2 - 1);
+  for (int i = tid; i < WV; i += D::THREADS) {
+    const int a = i % W, b = (i / W) % SM::W1, k = i / WW;
+    const int I = I0 + a, J = J0 + b, K = K0 + k;
+    const bool inr = I >= 0 && I < g.nv[0] && J >= 0 && J < g.nv[1] && K >= 0 && K < g.nv[2];
+    const long long node = inr ? I + (long long)g.nv[0] * (J + (long long)g.nv[1] * K) : 0;
+    const bool fcon = !raw && inr && !vmasked && face_constrained(g, I, J, K);
+    const int wi = widx(a, b, k);
 #pragma unroll
-      for (int cc = 0; cc < 3; ++cc) cp_async_3d(sx + cc * WVA + wi, A.xu + cc * Nv + node, inr && !fcon);
-      if (CONV) {  // v° as given (constrained nodes included)
+    for (int cc = 0; cc < 3; ++cc) cp_async_3d(sx + cc * WVA + wi, A.xu + cc * Nv + node, inr && !fcon);
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) cp_async_3d(svc + cc * WVA + wi, A.vc + cc * Nv + node, inr);
-      }
-      sflag[i] = (vmasked && inr) ? g.vmask[node] : 0;
-    }
+    for (int cc = 0; cc < 3; ++cc)  // v° as given (constrained nodes included)
+      cp_async_3d(svc + cc * WVA + wi, A.vc + cc * Nv + node, inr);
+    sflag[i] = (vmasked && inr) ? g.vmask[node] : 0;
   }
-  if (WBT) {
+  if (SADDLE) {
     const int P0 = cs0 - 1, Q0 = cs1 - 1, R0 = cs2 - 1;
     for (int i = tid; i < SM::PWV; i += D::THREADS) {
       const int P = P0 + i % PW0, Q = Q0 + (i / PW0) % SM::PW1, R = R0 + i / PW01;
@@ -166,7 +161,7 @@ __device__ __forceinline__ void tile3d_body(const TileArgs<T>& A, int bid) {
   for (int i = tid; i < SM::SU + SM::SP; i += D::THREADS) su[i] = T(0);
   asm volatile("cp.async.commit_group;\n" ::);
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  if (NEED_U && vmasked) {
+  if (vmasked) {
     for (int i = tid; i < WV; i += D::THREADS)
       if (sflag[i]) {
         const int wi = widx(i % W, (i / W) % SM::W1, i / WW);
@@ -219,55 +214,52 @@ __device__ __forceinline__ void tile3d_body(const TileArgs<T>& A, int bid) {
       for (int q = 0; q < 3; ++q)
 #pragma unroll
         for (int t = 0; t < 3; ++t) o[q][t] = fw(pa[q], 2 * lp[pa[q]] + t);
-      if (WU) {
-        T yl[27];
-        if (WA)
-          cell_A3p(sx + pa[0] * WVA, sx + pa[1] * WVA, sx + pa[2] * WVA, o[0], o[1], o[2], yl, eta, mmK, km_l, ex_l);
-        if (CONV && WA) {  // corrector stage: rho (C + S) on the thread's own component
-          const T* const vl[3] = {svc + pa[0] * WVA, svc + pa[1] * WVA, svc + pa[2] * WVA};
-          const T ihl[3] = {pa[0] == 0 ? A.ihx : (pa[0] == 1 ? A.ihy : A.ihz),
-                            pa[1] == 0 ? A.ihx : (pa[1] == 1 ? A.ihy : A.ihz),
-                            pa[2] == 0 ? A.ihx : (pa[2] == 1 ? A.ihy : A.ihz)};
-          cell_conv3<CONV>(sx + pa[0] * WVA, vl, o[0], o[1], o[2], A.rho, A.rk[cell], ihl, A.wq, yl);
+      T yl[27];
+      cell_A3p(sx + pa[0] * WVA, sx + pa[1] * WVA, sx + pa[2] * WVA, o[0], o[1], o[2], yl, eta, mmK, km_l, ex_l);
+      {  // rho (C + S) on the thread's own component
+        const T* const vl[3] = {svc + pa[0] * WVA, svc + pa[1] * WVA, svc + pa[2] * WVA};
+        const T ihl[3] = {pa[0] == 0 ? A.ihx : (pa[0] == 1 ? A.ihy : A.ihz),
+                          pa[1] == 0 ? A.ihx : (pa[1] == 1 ? A.ihy : A.ihz),
+                          pa[2] == 0 ? A.ihx : (pa[2] == 1 ? A.ihy : A.ihz)};
+        cell_conv3<CONV>(sx + pa[0] * WVA, vl, o[0], o[1], o[2], A.rho, A.rk[cell], ihl, A.wq, yl);
+      }
+      if (SADDLE) {
+        T pl[8];  // the cell's pressure nodes in the logical frame
+#pragma unroll
+        for (int lc = 0; lc < 2; ++lc)
+#pragma unroll
+          for (int lb = 0; lb < 2; ++lb)
+#pragma unroll
+            for (int la = 0; la < 2; ++la)
+              pl[la + 2 * lb + 4 * lc] =
+                  spw[fp(pa[0], lp[pa[0]] + la) + fp(pa[1], lp[pa[1]] + lb) + fp(pa[2], lp[pa[2]] + lc)];
+        cell_BT3p(pl, yl, bd_a);
+      }
+      int oo[3][3];
+      bool ok[3][3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          const int i = 2 * (lp[pa[q]] - 1) + t;
+          ok[q][t] = i >= 0 && i < vext[pa[q]];
+          oo[q][t] = fo(pa[q], i);
         }
-        if (WBT) {
-          T pl[8];  // the cell's pressure nodes in the logical frame
+      T* sc = su + comp * VSZA;
 #pragma unroll
-          for (int lc = 0; lc < 2; ++lc)
+      for (int lc = 0; lc < 3; ++lc) {
+        if (!ok[2][lc]) continue;
 #pragma unroll
-            for (int lb = 0; lb < 2; ++lb)
+        for (int lb = 0; lb < 3; ++lb) {
+          if (!ok[1][lb]) continue;
 #pragma unroll
-              for (int la = 0; la < 2; ++la)
-                pl[la + 2 * lb + 4 * lc] =
-                    spw[fp(pa[0], lp[pa[0]] + la) + fp(pa[1], lp[pa[1]] + lb) + fp(pa[2], lp[pa[2]] + lc)];
-          cell_BT3p(pl, yl, bd_a, WA);
-        }
-        int oo[3][3];
-        bool ok[3][3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-#pragma unroll
-          for (int t = 0; t < 3; ++t) {
-            const int i = 2 * (lp[pa[q]] - 1) + t;
-            ok[q][t] = i >= 0 && i < vext[pa[q]];
-            oo[q][t] = fo(pa[q], i);
-          }
-        T* sc = su + comp * VSZA;
-#pragma unroll
-        for (int lc = 0; lc < 3; ++lc) {
-          if (!ok[2][lc]) continue;
-#pragma unroll
-          for (int lb = 0; lb < 3; ++lb) {
-            if (!ok[1][lb]) continue;
-#pragma unroll
-            for (int la = 0; la < 3; ++la) {
-              if (!ok[0][la]) continue;
-              sc[oo[0][la] + oo[1][lb] + oo[2][lc]] += yl[la + 3 * lb + 9 * lc];
-            }
+          for (int la = 0; la < 3; ++la) {
+            if (!ok[0][la]) continue;
+            sc[oo[0][la] + oo[1][lb] + oo[2][lc]] += yl[la + 3 * lb + 9 * lc];
           }
         }
       }
-      if (WB && comp == 0) {  // comp 0: the rotated frame is the physical one
+      if (SADDLE && comp == 0) {  // comp 0: the rotated frame is the physical one
         T ob[8];
         cell_B3w(sx + 2 * lp[0], sx + WVA + 2 * lp[0], sx + 2 * WVA + 2 * lp[0], o[1], o[2], ob, c);
 #pragma unroll
@@ -292,37 +284,35 @@ __device__ __forceinline__ void tile3d_body(const TileArgs<T>& A, int bid) {
   }
 
   // ---- owned velocity nodes: epilogue ----
-  if (WU) {
-    const int nown = ve0 * ve1 * ve2;
-    for (int i = tid; i < nown; i += D::THREADS) {
-      const int i0 = i % ve0;
-      const int i1 = (i / ve0) % ve1;
-      const int i2 = i / (ve0 * ve1);
-      const int I = 2 * cs0 + i0, J = 2 * cs1 + i1, K = 2 * cs2 + i2;
-      const long long node = I + (long long)g.nv[0] * (J + (long long)g.nv[1] * K);
-      const bool con = !raw && vnode_constrained(g, node, I, J, K);
-      const int s = oidx(i0, i1, i2);
-      const int w = widx(i0 + 2, i1 + 2, i2 + 2);  // the node in the staged window
+  const int nown = ve0 * ve1 * ve2;
+  for (int i = tid; i < nown; i += D::THREADS) {
+    const int i0 = i % ve0;
+    const int i1 = (i / ve0) % ve1;
+    const int i2 = i / (ve0 * ve1);
+    const int I = 2 * cs0 + i0, J = 2 * cs1 + i1, K = 2 * cs2 + i2;
+    const long long node = I + (long long)g.nv[0] * (J + (long long)g.nv[1] * K);
+    const bool con = !raw && vnode_constrained(g, node, I, J, K);
+    const int s = oidx(i0, i1, i2);
+    const int w = widx(i0 + 2, i1 + 2, i2 + 2);  // the node in the staged window
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const long long gi = a * Nv + node;
-        const T ax = con ? (WA ? A.xu[gi] : T(0)) : su[a * VSZA + s];
-        if (MODE == TILE_APPLY) {
-          A.yu[gi] = ax;
-        } else if (MODE == TILE_RESID) {
-          A.yu[gi] = A.bu[gi] - ax;
-        } else {
-          const T r = A.bu[gi] - ax;
-          T dn = A.c2 * A.dinv[gi] * r;
-          if (A.use_d) dn += A.c1 * A.d[gi];
-          A.d[gi] = dn;
-          const T xin = (con || !NEED_U) ? A.xu[gi] : sx[a * WVA + w];
-          A.xout[gi] = xin + dn;
-        }
+    for (int a = 0; a < 3; ++a) {
+      const long long gi = a * Nv + node;
+      const T ax = con ? A.xu[gi] : su[a * VSZA + s];
+      if (MODE == TILE_APPLY) {
+        A.yu[gi] = ax;
+      } else if (MODE == TILE_RESID) {
+        A.yu[gi] = A.bu[gi] - ax;
+      } else {
+        const T r = A.bu[gi] - ax;
+        T dn = A.c2 * A.dinv[gi] * r;
+        if (A.use_d) dn += A.c1 * A.d[gi];
+        A.d[gi] = dn;
+        const T xin = con ? A.xu[gi] : sx[a * WVA + w];
+        A.xout[gi] = xin + dn;
       }
     }
   }
-  if (WB) {
+  if (SADDLE) {
     const int nown = pe0 * pe1 * pe2;
     for (int i = tid; i < nown; i += D::THREADS) {
       const int i0 = i % pe0;
@@ -330,7 +320,7 @@ __device__ __forceinline__ void tile3d_body(const TileArgs<T>& A, int bid) {
       const int i2 = i / (pe0 * pe1);
       const long long q = (cs0 + i0) + (long long)g.npn[0] * ((cs1 + i1) + (long long)g.npn[1] * (cs2 + i2));
       const bool con = !raw && pnode_constrained(g, q);
-      const T bx = con ? (WBT ? A.xp[q] : T(0)) : sp[i0 + D::PE0 * (i1 + D::PE1 * i2)];
+      const T bx = con ? A.xp[q] : sp[i0 + D::PE0 * (i1 + D::PE1 * i2)];
       if (MODE == TILE_RESID)
         A.yp[q] = A.bp[q] - bx;
       else
@@ -339,43 +329,40 @@ __device__ __forceinline__ void tile3d_body(const TileArgs<T>& A, int bid) {
   }
 }
 
-template <typename T, int MODE, bool WA, bool WBT, bool WB, int C2, int CONV = 0>
+template <typename T, int MODE, bool SADDLE, int CONV>
 struct TileK {
   using Args = TileArgs<T>;
-  using S = TileShape3<C2>;
-  static constexpr int THREADS = S::THREADS, MINB = 1;
-  static __device__ __forceinline__ void body(const Args& a, int blk, int) {
-    tile3d_body<T, MODE, WA, WBT, WB, S, CONV>(a, blk);
-  }
+  static constexpr int THREADS = TileShape3::THREADS, MINB = 1;
+  static __device__ __forceinline__ void body(const Args& a, int blk, int) { tile3d_body<T, MODE, SADDLE, CONV>(a, blk); }
 };
 
-template <typename T, int MODE, bool WA, bool WBT, bool WB, int C2, int CONV = 0>
-static cudaError_t launch_shape(TileArgs<T> a, cudaStream_t st) {
-  using S = TileShape3<C2>;
-  using SM = Smem3<T, MODE, WA, WBT, WB, S, CONV>;
+template <typename T, int MODE, bool SADDLE, int CONV>
+static cudaError_t launch_conv3(TileArgs<T> a, cudaStream_t st) {
+  using S = TileShape3;
+  using SM = Smem3<T, SADDLE>;
   a.tiles[0] = (a.g.n[0] + S::TC0 - 2) / (S::TC0 - 1);
   a.tiles[1] = (a.g.n[1] + S::TC1 - 2) / (S::TC1 - 1);
   a.tiles[2] = (a.g.n[2] + S::TC2 - 2) / (S::TC2 - 1);
   const size_t smem = sizeof(T) * SM::TOTAL + SM::FLAGS;
   const long long nblocks = (long long)a.tiles[0] * a.tiles[1] * a.tiles[2];
-  return submit<TileK<T, MODE, WA, WBT, WB, C2, CONV>>(a, nblocks, smem, st);
+  return submit<TileK<T, MODE, SADDLE, CONV>>(a, nblocks, smem, st);
 }
 
 template <typename T>
 cudaError_t launch_tile(int dim, int mode, int ops, TileArgs<T> a, cudaStream_t st) {
   if (mode == TILE_CHEB && ops != OPS_A) return cudaErrorInvalidValue;
   if (dim == 2) return launch_tile2d<T>(mode, ops, a, st);  // gs_tile2d.cu
-  if (a.conv && (ops & OPS_A)) {  // corrector stage: 8 x 8 x 4 halo tiles with the convection term
-    if (a.conv == 2) return mode == TILE_APPLY && ops == OPS_A ? launch_shape<T, TILE_APPLY, true, false, false, 4, 2>(a, st)
-                                                               : cudaErrorInvalidValue;
+  if (a.conv && (ops & OPS_A)) {  // corrector stage
+    if (a.conv == 2)
+      return mode == TILE_APPLY && ops == OPS_A ? launch_conv3<T, TILE_APPLY, false, 2>(a, st) : cudaErrorInvalidValue;
     if (ops == OPS_A) {
-      if (mode == TILE_APPLY) return launch_shape<T, TILE_APPLY, true, false, false, 4, 1>(a, st);
-      if (mode == TILE_RESID) return launch_shape<T, TILE_RESID, true, false, false, 4, 1>(a, st);
-      return launch_shape<T, TILE_CHEB, true, false, false, 4, 1>(a, st);
+      if (mode == TILE_APPLY) return launch_conv3<T, TILE_APPLY, false, 1>(a, st);
+      if (mode == TILE_RESID) return launch_conv3<T, TILE_RESID, false, 1>(a, st);
+      return launch_conv3<T, TILE_CHEB, false, 1>(a, st);
     }
     if (ops == (OPS_A | OPS_BT | OPS_B)) {
-      if (mode == TILE_APPLY) return launch_shape<T, TILE_APPLY, true, true, true, 4, 1>(a, st);
-      if (mode == TILE_RESID) return launch_shape<T, TILE_RESID, true, true, true, 4, 1>(a, st);
+      if (mode == TILE_APPLY) return launch_conv3<T, TILE_APPLY, true, 1>(a, st);
+      if (mode == TILE_RESID) return launch_conv3<T, TILE_RESID, true, 1>(a, st);
     }
     return cudaErrorInvalidValue;
   }
