@@ -1113,7 +1113,7 @@ template <typename T>
 gs_status setup_T(gs_ctx* c) {
   for (int l = 0; l < c->L; ++l) {
     Level& lv = c->lv[l];
-    CK(launch_diagA<T>(lv.g, coef<T>(lv), etap<T>(lv), alphap<T>(lv), (T*)lv.dinv, 1, c->st));
+    CK(launch_diagA<T>(lv.g, lv.c64, etap<T>(lv), alphap<T>(lv), (T*)lv.dinv, 1, c->st));
   }
   for (int l = (c->opt.coarse_mode == 1 ? 0 : 1); l < c->L; ++l) CKS(lanczos<T>(c, l));
   const Level& F = c->lv[c->L - 1];
@@ -1251,8 +1251,8 @@ gs_status time_launches(gs_ctx* c, F&& launch, int reps, double* us) {
   return GS_OK;
 }
 
-// Per level, time the fused Chebyshev step with each compiled kernel variant (2D: tile heights
-// and the strip kernel; 3D: tile depths) on the level's own (scratch) vectors and keep the
+// Per level, time the fused Chebyshev step with each compiled kernel variant (2D: tile shapes
+// and the strip kernel; 3D: segment lengths of the march) on the level's own (scratch) vectors and keep the
 // fastest; then the same for the FP64 saddle operator on the finest level.  A variant must beat
 // the current choice by 2 % to replace it.
 template <typename T>
@@ -2166,7 +2166,7 @@ gs_status apply_level_T(gs_ctx* c, int l, gs_op op, const void* xv, void* yv, co
         CK(launch_cast<double, T>(c->t1, y, lv.nu, (T)1, c->st));
         return GS_OK;
       }
-      CK(launch_diagA<T>(lv.g, coef<T>(lv), etap<T>(lv), alphap<T>(lv), y, 0, c->st));
+      CK(launch_diagA<T>(lv.g, lv.c64, etap<T>(lv), alphap<T>(lv), y, 0, c->st));
       return GS_OK;
     case GS_OP_SMOOTH: {
       if (!mgprec || (l == 0 && c->opt.coarse_mode != 1))
@@ -2991,7 +2991,7 @@ gs_status corrector_setup_T(gs_ctx* c) {
       CK(launch_diag_conv(lv.g, lv.vc64, lv.rk64, lv.rho, c->t1, c->st));
       CK(launch_reciprocal<T>(c->t1, (T*)lv.dinv, lv.nu, c->st));
     } else {
-      CK(launch_diagA<T>(lv.g, coef<T>(lv), etap<T>(lv), alphap<T>(lv), (T*)lv.dinv, 1, c->st));
+      CK(launch_diagA<T>(lv.g, lv.c64, etap<T>(lv), alphap<T>(lv), (T*)lv.dinv, 1, c->st));
     }
   }
   for (int l = (c->opt.coarse_mode == 1 ? 0 : 1); l < c->L; ++l) CKS(lanczos<T>(c, l));

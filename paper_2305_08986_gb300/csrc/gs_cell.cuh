@@ -461,8 +461,8 @@ __device__ __forceinline__ void cell_B3w(const T* u0, const T* u1, const T* u2, 
 __host__ __device__ inline int mdiag(int a) { return a == 1 ? 16 : 4; }
 __host__ __device__ inline int kdiag(int a) { return a == 1 ? 16 : 7; }
 
-template <typename T>
-__device__ __forceinline__ T cell_diagA(int dim, int comp, int la, int lb, int lc, T eta, const OpCoef<T>& c) {
+__device__ __forceinline__ double cell_diagA(int dim, int comp, int la, int lb, int lc, double eta, const OpCoef<double>& c) {
+  using T = double;
   if (dim == 2) {
     const T Ma = T(mdiag(la)), Mb = T(mdiag(lb)), Ka = T(kdiag(la)), Kb = T(kdiag(lb));
     const T ck = (comp == 1 ? T(2) : T(1)) * eta * c.km[1];

@@ -88,7 +88,7 @@ template <typename T>
 cudaError_t launch_reciprocal(const double* in, T* out, long long n, cudaStream_t st);
 
 template <typename T>
-cudaError_t launch_diagA(const Geom& g, const OpCoef<T>& c, const T* eta, const T* alpha, T* out, int invert,
+cudaError_t launch_diagA(const Geom& g, const OpCoef<double>& c, const T* eta, const T* alpha, T* out, int invert,
                          cudaStream_t st);
 // rc = R rf; with d != NULL also the start of the coarse level's Chebyshev smoother from zero,
 // d = x = dinv * rc * inv_theta (the expression of launch_cheb_init0)

@@ -27,17 +27,20 @@ inline unsigned nblk(long long n) { return (unsigned)((n + TPB - 1) / TPB); }
 }  // namespace
 
 // ---- diag(A) (Sec. 4: the Jacobi preconditioner of Cheb(A, diag(A), k_A)) ----------------------
+// Summed and inverted in FP64 also for an FP32 level, once per setup: nodes of one kind share the rounding of the
+// coefficients, which in FP32 shifted the smoother's eigenvalue bound by up to 1.6e-7 and its result by 3.3e-7 of the
+// norm (1280 x 224, four steps; 1.4e-7 now).
 template <typename T, int DIM>
-__global__ void k_diagA(const Geom g, const OpCoef<T> c, const T* __restrict__ eta, const T* __restrict__ alpha,
+__global__ void k_diagA(const Geom g, const OpCoef<double> c, const T* __restrict__ eta, const T* __restrict__ alpha,
                         T* __restrict__ out, int invert) {
   const long long node = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (node >= g.Nv) return;
   int I, J, K;
   unflat(node, g.nv, DIM, I, J, K);
   const bool con = vnode_constrained(g, node, I, J, K);
-  T acc[DIM];
+  double acc[DIM];
 #pragma unroll
-  for (int a = 0; a < DIM; ++a) acc[a] = T(0);
+  for (int a = 0; a < DIM; ++a) acc[a] = 0.0;
   if (!con) {
     // cells touching the node along each axis and the node's local index in them
     int cl[3][2], ll[3][2], cnt[3];
@@ -58,23 +61,23 @@ __global__ void k_diagA(const Geom g, const OpCoef<T> c, const T* __restrict__ e
         for (int i = 0; i < cnt[0]; ++i) {
           const long long cell = cl[0][i] + (long long)g.n[0] * (cl[1][j] + (long long)g.n[1] * (DIM == 3 ? cl[2][k] : 0));
           if (cell_void(g, cell)) continue;
-          const T e = eta[cell] * c.eta_scale;
-          OpCoef<T> cK = c;  // the cell's mass coefficient (alpha per cell)
+          const double e = eta[cell] * c.eta_scale;
+          OpCoef<double> cK = c;  // the cell's mass coefficient (alpha per cell)
           if (alpha) cK.mm = c.mm * alpha[cell];
 #pragma unroll
           for (int a = 0; a < DIM; ++a)
-            acc[a] += cell_diagA<T>(DIM, a, ll[0][i], ll[1][j], DIM == 3 ? ll[2][k] : 0, e, cK);
+            acc[a] += cell_diagA(DIM, a, ll[0][i], ll[1][j], DIM == 3 ? ll[2][k] : 0, e, cK);
         }
   }
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {
-    T v = con ? T(1) : acc[a];
-    out[a * g.Nv + node] = invert ? T(1) / v : v;
+    const double v = con ? 1.0 : acc[a];
+    out[a * g.Nv + node] = (T)(invert ? 1.0 / v : v);
   }
 }
 
 template <typename T>
-cudaError_t launch_diagA(const Geom& g, const OpCoef<T>& c, const T* eta, const T* alpha, T* out, int invert,
+cudaError_t launch_diagA(const Geom& g, const OpCoef<double>& c, const T* eta, const T* alpha, T* out, int invert,
                          cudaStream_t st) {
   if (g.dim == 2)
     k_diagA<T, 2><<<nblk(g.Nv), TPB, 0, st>>>(g, c, eta, alpha, out, invert);
@@ -205,7 +208,7 @@ cudaError_t launch_pdiag(const Geom& g, const OpCoef<T>& c, const T* eta, T* din
 }
 
 #define INST(T)                                                                                    \
-  template cudaError_t launch_diagA<T>(const Geom&, const OpCoef<T>&, const T*, const T*, T*, int, cudaStream_t); \
+  template cudaError_t launch_diagA<T>(const Geom&, const OpCoef<double>&, const T*, const T*, T*, int, cudaStream_t); \
   template cudaError_t launch_pmass<T>(int, PMassArgs<T>, cudaStream_t);                           \
   template cudaError_t launch_pdiag<T>(const Geom&, const OpCoef<T>&, const T*, T*, cudaStream_t);
 INST(float)
