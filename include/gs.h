@@ -342,7 +342,8 @@ typedef struct {
   int pressure_coarse_free;/* unknowns of the dense coarse pressure-Laplacian solve */
   double plambda_max[16];  /* Chebyshev upper bound of the pressure Laplacian per level */
   int tile_rows[16];       /* 2D: evaluated cell rows per tile chosen for each level's multigrid kernels
-                              (0: the strip kernel); 3D: 4 for segments of at most 4 evaluated cell
+                              (0: the strip kernel; 8: tiles of 32 x 8 or of 8 x 8 cells, which this field
+                              does not tell apart); 3D: 4 for segments of at most 4 evaluated cell
                               layers, 8 for segments of the length chosen by size */
   int saddle_tile_rows;    /* the same for the FP64 saddle operator */
   int deflation_inclusions;/* stiff inclusions in the deflation space (option deflate) */

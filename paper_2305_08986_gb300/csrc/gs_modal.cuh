@@ -115,10 +115,10 @@ __device__ __forceinline__ void from_modes2(f32x2& r0, f32x2& r1, f32x2& r2) {
   r1 = y1;
 }
 // y = (alpha_K M + eta_K viscous) x of one 2D cell in FP32, the two components in the halves of pairs: the sums of
-// cell_modal2 with the same roundings (the same bits) in about 90 instead of 150 instructions.  For the strip
-// kernel, which is bound by instruction issue: A x 1280 x 210 7.74 -> 7.48 us, smoother call 1280 x 224 58.8 -> 57.1
-// us.  The tile kernels of small meshes are bound by latency and keep the scalar form (32 x 32 smoother call: 16.1
-// us, 16.4 us with pairs).
+// cell_modal2 with the same roundings (the same bits) in about 100 instead of 165 instructions.  For the strip kernel: A x
+// 1280 x 210 7.74 -> 7.48 us, smoother call 1280 x 224 58.8 -> 57.1 us; small gains, because it waits for its staged rows
+// and barriers more than it issues (51 % of the issue slots).  The tile kernels of small meshes keep the scalar form
+// (32 x 32 smoother call: 16.1 us, 16.4 us with pairs).
 __device__ __forceinline__ void cell_modal2_pair(const float (&x)[2][9], float (&y)[2][9], float eta, float alpha,
                                                  const Modal2<float>& m) {
   f32x2 v[9];
