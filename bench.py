@@ -271,11 +271,10 @@ def run_reference(args, rank, world):
 # --------------------------------------------------------------------------------------------
 # GPU arm
 # --------------------------------------------------------------------------------------------
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, from one ncu --set full
-# capture of each kernel as built now: the finest-level fused Chebyshev step at the 1280 x 224
-# workload (strip kernel; its writes d, x' stay in L2 within the capture, so the figure is the read
-# traffic) and the FP64 saddle operator (x and eta read once; y and spilled registers written).
-NCU_TRAFFIC_BYTES = {"cheb_step": 38.5664e6 + 7.936e3, "saddle_fp64": 25.351168e6 + 7.776256e6}
+# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch at the 1280 x 224 workload, from one ncu
+# capture of each kernel with its cells in Legendre modes: the finest-level fused Chebyshev step (strip kernel) and the
+# FP64 saddle operator.  Their results stay in L2 within the capture, so the figures are the read traffic.
+NCU_TRAFFIC_BYTES = {"cheb_step": 38.564096e6 + 1.536e3, "saddle_fp64": 24.745216e6 + 1.024e3}
 
 
 def tile_step_bytes(n_u: int, n_cells: int, elem: int, kind: str) -> int:

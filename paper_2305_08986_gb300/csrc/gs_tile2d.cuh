@@ -390,8 +390,8 @@ struct Tile2dK {
   // FP64 with B^T (the saddle operator, FP64-pipe-bound): 3 CTAs per SM.  1280 x 224: 134 us with the cells in
   // Legendre modes, 260 us in 3 x 3 sweeps (about 400 FP64 instructions per cell).  In modes an evaluated cell takes 181
   // (to modes 48, A 53, B^T 16, B 16, back to nodes 48) and the node sums 13 per owned cell; 32 x 8
-  // tiles evaluate 1.18 cells per cell, so 226 in all: 103 us on a pipe of 2 per SM and clock.  The FP32 variants stay
-  // at 2
+  // tiles evaluate 1.18 cells per cell, so 226 in all (225 counted): 102 us on a pipe of 2 per SM and clock, which is
+  // busy 81 % of the time.  The FP32 variants stay at 2
   static constexpr int THREADS = S2::NT, MINB = CONV ? 1 : (S2::E0 == 8 ? 8 : (sizeof(T) == 8 && WBT ? 3 : 2));
   static __device__ __forceinline__ void body(const Args& a, int blk, int) {
     tile2d_body<T, S2, MODE, WA, WBT, WB, CONV>(a, blk);
